@@ -257,6 +257,10 @@ KParams make_kparams(const starkv_state* st) {
   k.decay_mode = c.decay_mode;
   k.aeb_mode = c.aeb_mode;
   k.mi_span = c.mi_span;
+  auto reciprocal = [](int n) { return n > 1 ? static_cast<uint32_t>(((uint64_t(1) << 32) + n - 1) / n) : 0u; };
+  k.inv_K = reciprocal(k.K);
+  k.inv_R = reciprocal(k.R);
+  k.inv_C = reciprocal(k.C);
   k.wait_ns = st->wait_ns;
   return k;
 }
@@ -264,7 +268,7 @@ KParams make_kparams(const starkv_state* st) {
 // Workspace regions of one call over layers [layer0, layer0 + nlayers).
 struct WsPlan {
   size_t partials = 0, s_raw = 0, total = 0;
-  std::vector<size_t> raw_off, S_off, score_off, vis_off;  // per seq, SIZE_MAX = not in workspace
+  std::vector<size_t> raw_off, S_off, score_off;  // per seq, SIZE_MAX = not in workspace
 };
 
 int tiles_of(int lp) { return (lp + kTileKeys - 1) / kTileKeys; }
@@ -276,13 +280,11 @@ size_t sel_rows(const starkv_config& c) {
 
 size_t stats_bytes(const starkv_config& c) { return static_cast<size_t>(STARKV_STATS_STRIDE(c.n_kv_heads)) * 4; }
 
-// ws_score: the calibration kernel runs (fused score region; key/cell region
-// of the rows longer than its shared-memory capacity).
+// ws_score: the calibration kernel runs (fused score region).
 void plan_ws(const starkv_state* st, const starkv_seq* seqs, int nseq, int nlayers, bool ws_S,
              bool ws_score, WsPlan* p) {
   const starkv_config& c = st->cfg;
   const int G = c.n_kv_heads;
-  const int cap = calibrate_capacity(c.mi_bins, c.mi_grid, c.grid_rows, c.grid_cols);
   size_t off = 0;
   size_t tiles = 0;
   for (int i = 0; i < nseq; ++i) tiles += static_cast<size_t>(nlayers) * G * tiles_of(seqs[i].L - c.window);
@@ -291,15 +293,10 @@ void plan_ws(const starkv_state* st, const starkv_seq* seqs, int nseq, int nlaye
   p->raw_off.assign(nseq, SIZE_MAX);
   p->S_off.assign(nseq, SIZE_MAX);
   p->score_off.assign(nseq, SIZE_MAX);
-  p->vis_off.assign(nseq, SIZE_MAX);
   for (int i = 0; i < nseq; ++i) {
     const size_t lp = seqs[i].L - c.window;
-    if (ws_score && lp > static_cast<size_t>(cap)) {
-      p->vis_off[i] = off;
-      off += align256(static_cast<size_t>(nlayers) * G * lp * 3 * sizeof(uint32_t));
-    }
     p->raw_off[i] = off;
-    off += align256(static_cast<size_t>(nlayers) * G * kRawCopies * raw_stride(static_cast<int>(lp)) * sizeof(float));
+    off += align256(static_cast<size_t>(nlayers) * G * raw_stride(static_cast<int>(lp)) * sizeof(float));
     if (ws_S && !seqs[i].S) {
       p->S_off[i] = off;
       off += align256(static_cast<size_t>(c.n_layers) * G * lp * sizeof(float));
@@ -334,7 +331,6 @@ SeqView make_view(const starkv_state* st, const starkv_seq& s, char* ws, const W
   v.s_raw = reinterpret_cast<float*>(ws + plan.raw_off[i]);
   v.score = plan.score_off[i] != SIZE_MAX ? reinterpret_cast<float*>(ws + plan.score_off[i]) : s.score;
   v.stats = s.stats;
-  v.vis = plan.vis_off[i] != SIZE_MAX ? reinterpret_cast<uint32_t*>(ws + plan.vis_off[i]) : nullptr;
   return v;
 }
 
@@ -454,7 +450,7 @@ starkv_status run_stages(starkv_state* st, const starkv_seq* seqs, int nseq, int
       }));
     if (stages & kSelect)
       CUDA_TRY(launch(st, STARKV_KERNEL_CALIBRATE, stream, [&] {
-        return calibrate_launch(b, kp, st->dev, (stages & kStatsRaw) != 0, lp_max, stream);
+        return calibrate_launch(b, kp, st->dev, (stages & kStatsRaw) != 0, lp_max, st->num_sms, stream);
       }));
     if ((stages & kCompact) && rows_out_max > 0)
       CUDA_TRY(launch(st, STARKV_KERNEL_COMPACT, stream, [&] {
@@ -639,9 +635,7 @@ starkv_status starkv_init_state(const starkv_config* cfg, starkv_state** out, vo
   const size_t G = cfg->n_kv_heads, RC = static_cast<size_t>(cfg->grid_rows) * cfg->grid_cols;
   const size_t o_n = 0;
   const size_t o_mibar = o_n + align256(SL * sizeof(int32_t));
-  const size_t o_micur = o_mibar + align256(SL * G * sizeof(double));
-  const size_t o_phi = o_micur + align256(SL * G * sizeof(double));
-  const size_t o_m = o_phi + align256(SL * G * sizeof(float));
+  const size_t o_m = o_mibar + align256(SL * G * sizeof(double));
   const size_t o_err = o_m + align256(SL * G * RC * sizeof(float));
   st->mem_bytes = o_err + 256;
   e = cudaMalloc(&st->mem, st->mem_bytes);
@@ -652,8 +646,6 @@ starkv_status starkv_init_state(const starkv_config* cfg, starkv_state** out, vo
   char* m = static_cast<char*>(st->mem);
   st->dev.n = reinterpret_cast<int32_t*>(m + o_n);
   st->dev.mi_bar = reinterpret_cast<double*>(m + o_mibar);
-  st->dev.mi_cur = reinterpret_cast<double*>(m + o_micur);
-  st->dev.phi_cur = reinterpret_cast<float*>(m + o_phi);
   st->dev.m = reinterpret_cast<float*>(m + o_m);
   st->dev.err = reinterpret_cast<uint32_t*>(m + o_err);
   e = cudaMemsetAsync(st->mem, 0, st->mem_bytes, static_cast<cudaStream_t>(stream));

@@ -19,7 +19,6 @@ constexpr int kMaxBatch = 32;       // sequences per launch (kernel-parameter ar
 constexpr int kMaxBins = 64;        // K rank bins
 constexpr int kMaxHist = 4096;      // K * M^2
 constexpr int kMaxGrid = 16384;     // R * C
-constexpr int kRawCopies = 4;       // unpooled group sums: one copy per pass-2 column quarter
 
 // device error word bits
 constexpr uint32_t kErrTimeout = 1u;
@@ -37,8 +36,6 @@ struct DevState {
   int32_t* n;          // [slots][layers] steps seen
   double* mi_bar;      // [slots][layers][G] MI EMA (Eq. 6)
   float* m;            // [slots][layers][G][R*C] temporal EMA m_g (Eq. 8)
-  double* mi_cur;      // [slots][layers][G] MI of the current step (group_stats -> select)
-  float* phi_cur;      // [slots][layers][G] phi_g of the current step
   uint32_t* err;       // device error word
 };
 
@@ -50,6 +47,8 @@ struct KParams {
   int decay_mode;      // 0 exponential (Eq. 9), 1 linear, 2 power law
   int aeb_mode;        // 0 entropy (Sec. 3.6), 1 peak confidence
   int mi_span;         // 0 every historical visual token, 1 the newest frame's
+  uint32_t inv_K, inv_R, inv_C;   // ceil(2^32 / n), 0 for n = 1: x / n = high word of x * inv for x < 2^28, n <= 16
+                                  // (and x < 2^16, n <= 1024)
   uint64_t wait_ns;    // bounded-wait limit
 };
 
@@ -66,11 +65,9 @@ struct SeqView {
   uint32_t* meta_out;
   int32_t* idx;    // [n_layers][P][B]
   float* S;        // [n_layers][G][Lp] (a workspace region when the caller passed NULL)
-  float* s_raw;    // [n_layers_in_launch][G][kRawCopies][raw_stride(Lp)] unpooled sums (workspace) or NULL
+  float* s_raw;    // [n_layers_in_launch][G][raw_stride(Lp)] unpooled sums (workspace) or NULL
   float* score;    // [n_layers][P][Lp] fused score, P = 1 or G (a workspace region when NULL)
   float* stats;    // optional
-  uint32_t* vis;   // [n_layers_in_launch][G][3 Lp] keys, candidate list and cells of
-                   // rows too long for shared memory (workspace), else NULL
 };
 
 struct SeqBatch {

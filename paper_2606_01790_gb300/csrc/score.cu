@@ -51,6 +51,8 @@ constexpr int kEpiThreads = 32 * kEpiWarps;
 constexpr uint32_t kFull = 0xffffffffu;
 constexpr int kXOnesBytes = 256;              // pass 2: the ones operand (two 8 x 16 B core matrices)
 constexpr int kXRowBytes = 32;                // pass 2: one window row of the -lse operand (16 bf16)
+constexpr int kSumSlots = 8;                  // pass 2: tiles whose column-quarter sums are kept (see k_score_accum)
+constexpr int kSumBytes = kSumSlots * 4 * kTileKeys * 4;
 // Limit of the waits for copies and MMAs this CTA has already issued, before
 // it exits or releases TMEM: those complete in microseconds, so the limit only
 // guards against a broken memory system, whatever the configured wait limit.
@@ -543,8 +545,10 @@ __global__ void __launch_bounds__(kScoreThreads, 1) k_score_accum(const __grid_c
   uint8_t* sQ = smem;                          // [2 halves][q_rows][128 B]
   uint8_t* sK = smem + 2 * p.q_rows * 128;     // [kstages][2 halves][128][128 B]
   SmemCtl* ctl = reinterpret_cast<SmemCtl*>(sK + p.kstages * kTileBytes);
-  // ones operand [256 B], then two buffers of the -lse operand [q_rows][32 B]
+  // ones operand [256 B], then two buffers of the -lse operand [q_rows][32 B],
+  // then [kSumSlots][4 column quarters][128 keys] sums of the last tiles
   uint8_t* sX = reinterpret_cast<uint8_t*>(ctl) + 256;
+  float* sS = reinterpret_cast<float*>(sX + kXOnesBytes + 2 * p.q_rows * kXRowBytes);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
   if (threadIdx.x == 0) ctl_init(ctl, p.kstages);
@@ -606,8 +610,22 @@ __global__ void __launch_bounds__(kScoreThreads, 1) k_score_accum(const __grid_c
     };
     int jt = 0, kp = 0;
     bool dead = false;
-    float* dst = nullptr;   // this thread's copy of the piece's unpooled row
+    float* dst = nullptr;   // the piece's unpooled row, at this thread's key of tile 0
     int lp = 0;
+    // The four column quarters of a key lie in four warps.  Each writes its
+    // sum of tile j to slot j mod 8 before it releases the tile's accumulator
+    // stage, so that a warp that finds tile j + 2 ready (the stage's next
+    // product, issued once all 16 warps had released it) finds all four: one
+    // warp of each lane quadrant, in turn, then adds them in order and stores
+    // the row.  No warp waits for another, and one row goes to memory instead
+    // of four.  A slot is written again at tile j + 8, after every warp has
+    // released tile j + 6 and so read the slot long before.
+    float *pend1 = nullptr, *pend2 = nullptr;   // where this key's sums of the last two tiles go (NULL: past the row)
+    auto flush = [&](int j, float* to) {   // tile j's sums, by warpgroup j mod 4
+      if ((j & 3) != wg || to == nullptr) return;
+      const float* v = sS + (j & (kSumSlots - 1)) * (4 * kTileKeys) + q;
+      *to = ((v[0] + v[kTileKeys]) + v[2 * kTileKeys]) + v[3 * kTileKeys];
+    };
     TileIter c;
     c.init(p, fb, fe);
     if (c.valid()) {
@@ -633,7 +651,7 @@ __global__ void __launch_bounds__(kScoreThreads, 1) k_score_accum(const __grid_c
         ++kp;
         const ScoreSeq& sq = p.seq[c.s];
         lp = sq.Lp;
-        dst = sq.s_raw + (static_cast<int64_t>(c.l * p.G + c.g) * kRawCopies + wg) * raw_stride(lp) + q;
+        dst = sq.s_raw + static_cast<int64_t>(c.l * p.G + c.g) * raw_stride(lp) + q;
       }
       const int ts = jt & 1;
       if (!dead) {
@@ -645,15 +663,23 @@ __global__ void __launch_bounds__(kScoreThreads, 1) k_score_accum(const __grid_c
           float2 a0 = make_float2(0.f, 0.f), a1 = make_float2(0.f, 0.f);
           if (nch > 0)
             stream16(base0 + ts * 256, nch, [&](const uint32_t(&v)[16], int) { exp2_acc16(v, sc2, zero2, a0, a1); });
+          const float2 a = fadd2(a0, a1);
+          sS[((jt & (kSumSlots - 1)) * 4 + wg) * kTileKeys + q] = a.x + a.y;
           tc_fence_before();
           __syncwarp();
           if (lane == 0) mbar_arrive(&ctl->t_empty[ts]);
+          if (jt >= 2) flush(jt - 2, pend2);
           const int key0 = c.j * kTileKeys;
-          const float2 a = fadd2(a0, a1);
-          if (key0 + q < lp) dst[key0] = a.x + a.y;
+          pend2 = pend1;
+          pend1 = key0 + q < lp ? dst + key0 : nullptr;
         }
       }
       ++jt;
+    }
+    named_bar_sync(1, kEpiThreads);   // every warp's last sums are written (all reach this, also after a timeout)
+    if (!dead) {
+      if (jt >= 2) flush(jt - 2, pend2);
+      if (jt >= 1) flush(jt - 1, pend1);
     }
   }
   __syncthreads();
@@ -664,7 +690,7 @@ __global__ void __launch_bounds__(kScoreThreads, 1) k_score_accum(const __grid_c
 }
 
 // S[g, t] = (G/H)(1/k) sum_{|j| <= k/2} S_raw[g, t + j]  (Eqs. 3-4; zero padding,
-// divisor k), S_raw being the sum of its column-quarter copies.  grid: (ceil(Lp_max / 256), nlayers * G, nseq)
+// divisor k).  grid: (ceil(Lp_max / 256), nlayers * G, nseq)
 __global__ void k_pool(const __grid_constant__ SeqBatch b, int G, int H, int pool) {
   griddep_launch_dependents();
   griddep_wait();
@@ -673,26 +699,21 @@ __global__ void k_pool(const __grid_constant__ SeqBatch b, int G, int H, int poo
   if (t >= s.Lp) return;
   const int lg = blockIdx.y;                  // launch-local layer * G + g
   const int layer = b.layer0 + lg / G, g = lg % G;
-  const int rs = raw_stride(s.Lp);
-  const float* src = s.s_raw + static_cast<int64_t>(lg) * kRawCopies * rs;
+  const float* src = s.s_raw + static_cast<int64_t>(lg) * raw_stride(s.Lp);
   const int half = pool >> 1;
   float acc = 0.f;
   for (int j = -half; j <= half; ++j) {
     const int u = t + j;
-    if (u >= 0 && u < s.Lp) {
-      float r = 0.f;
-      for (int c = 0; c < kRawCopies; ++c) r += src[c * rs + u];
-      acc += r;
-    }
+    if (u >= 0 && u < s.Lp) acc += src[u];
   }
   const float scale = static_cast<float>(G) / static_cast<float>(H) / static_cast<float>(pool);
   s.S[(static_cast<int64_t>(layer) * G + g) * s.Lp + t] = acc * scale;
 }
 
 // alignment slack + Q + K stages + control block + the larger of the pass-1
-// merge buffer and the pass-2 -lse operands (ones + two row buffers)
+// merge buffer and pass 2's -lse operands (ones + two row buffers) and sums
 size_t score_smem_bytes(int q_rows, int kstages) {
-  const size_t aux = std::max<size_t>(4 * 128 * sizeof(float2), kXOnesBytes + 2 * static_cast<size_t>(q_rows) * kXRowBytes);
+  const size_t aux = std::max<size_t>(4 * 128 * sizeof(float2), kXOnesBytes + 2 * static_cast<size_t>(q_rows) * kXRowBytes + kSumBytes);
   return 1024 + static_cast<size_t>(2 * q_rows * 128) + static_cast<size_t>(kstages) * kTileBytes + 256 + aux;
 }
 
