@@ -84,40 +84,42 @@ __device__ __forceinline__ TileCoord decode(const ScoreParams& p, int64_t f) {
 
 __device__ __forceinline__ int64_t range_begin(int64_t T, int c, int P) { return T * c / P; }
 
-// Coordinates of consecutive flat tiles [f0, f1), advanced without divisions
-// (one decode at the start).  A piece is a run of tiles of one (seq, layer,
-// group) row inside the range.
-struct TileIter {
-  int s, l, g, j, nt;
-  int64_t f, fe;
-  __device__ void init(const ScoreParams& p, int64_t f0, int64_t f1) {
-    f = f0;
-    fe = f1;
-    s = l = g = j = nt = 0;
-    if (f >= fe) return;
+// The pieces of a CTA's flat range [f0, f1), in order: a piece is a run of n
+// tiles j0, j0 + 1, ... of one (seq, layer, group) row, f its first flat tile.
+// One decode at the start, no divisions after it, and nothing but a counter
+// inside a piece: the tile loops of the four roles carry no coordinates.
+struct PieceIter {
+  int s, l, g, j0, n, nt;
+  int rem;        // tiles of the range from this piece on
+  int64_t f;
+  __device__ __forceinline__ PieceIter(const ScoreParams& p, int64_t f0, int64_t f1)
+      : s(0), l(0), g(0), j0(0), n(0), nt(0), rem(static_cast<int>(f1 - f0)), f(f0) {
+    if (rem <= 0) return;
     const TileCoord c = decode(p, f0);
     s = c.s;
     l = c.l;
     g = c.g;
-    j = c.j;
+    j0 = c.j;
     nt = p.seq[s].nt;
+    n = min(rem, nt - j0);
   }
-  __device__ bool valid() const { return f < fe; }
-  __device__ bool first(int64_t fb) const { return f == fb || j == 0; }
-  __device__ bool last() const { return f + 1 == fe || j + 1 == nt; }
-  __device__ void next(const ScoreParams& p) {
-    ++f;
-    if (f >= fe) return;
-    if (++j < nt) return;
-    j = 0;
-    if (++g < p.G) return;
-    g = 0;
-    if (++l < p.nlayers) return;
-    l = 0;
-    do {
-      ++s;
-    } while (s + 1 < p.nseq && p.seq[s].nt == 0);
-    nt = p.seq[s].nt;
+  __device__ __forceinline__ bool valid() const { return rem > 0; }
+  __device__ __forceinline__ void next(const ScoreParams& p) {
+    f += n;
+    rem -= n;
+    j0 = 0;
+    if (rem <= 0) return;
+    if (++g == p.G) {
+      g = 0;
+      if (++l == p.nlayers) {
+        l = 0;
+        do {
+          ++s;
+        } while (s + 1 < p.nseq && p.seq[s].nt == 0);
+        nt = p.seq[s].nt;
+      }
+    }
+    n = min(rem, nt);
   }
 };
 
@@ -174,36 +176,35 @@ __device__ void producer_loop(const ScoreParams& p, SmemCtl* ctl, uint8_t* sQ, u
   int last_q_pc = -1;
   int last_ph[kMaxStages];
   for (int i = 0; i < kMaxStages; ++i) last_ph[i] = -1;
-  TileIter c;
-  for (c.init(p, fb, fe); c.valid(); c.next(p)) {
-    if (ctl->abort) break;
-    if (c.first(fb)) {
-      if (!mbar_wait(&ctl->q_empty, (pc & 1) ^ 1, p.wait_ns)) { fail(ctl, p.err); break; }
-      const int zq = p.layer0 + c.l, y = c.g * p.rows;
-      if (PASS == 1) {
-        mbar_arrive_expect_tx(&ctl->q_full, p.rows * 256);
-        for (int h = 0; h < 2; ++h) {
-          tma_load_3d(sQ + h * qhalf, &p.tmqa[c.s], &ctl->q_full, h * 64, y, zq);
-          if (p.rows > kTileKeys)
-            tma_load_3d(sQ + h * qhalf + kTileKeys * 128, &p.tmqb[c.s], &ctl->q_full, h * 64, y + kTileKeys, zq);
-        }
-      } else {
-        mbar_arrive_expect_tx(&ctl->q_full, p.n2 * 256);
-        for (int h = 0; h < 2; ++h) tma_load_3d(sQ + h * qhalf, &p.tmq2[c.s], &ctl->q_full, h * 64, y, zq);
+  for (PieceIter c(p, fb, fe); c.valid() && !ctl->abort; c.next(p)) {
+    if (!mbar_wait(&ctl->q_empty, (pc & 1) ^ 1, p.wait_ns)) { fail(ctl, p.err); break; }
+    const int zq = p.layer0 + c.l, y = c.g * p.rows;
+    if (PASS == 1) {
+      mbar_arrive_expect_tx(&ctl->q_full, p.rows * 256);
+      for (int h = 0; h < 2; ++h) {
+        tma_load_3d(sQ + h * qhalf, &p.tmqa[c.s], &ctl->q_full, h * 64, y, zq);
+        if (p.rows > kTileKeys)
+          tma_load_3d(sQ + h * qhalf + kTileKeys * 128, &p.tmqb[c.s], &ctl->q_full, h * 64, y + kTileKeys, zq);
       }
-      last_q_pc = pc;
-      ++pc;
+    } else {
+      mbar_arrive_expect_tx(&ctl->q_full, p.n2 * 256);
+      for (int h = 0; h < 2; ++h) tma_load_3d(sQ + h * qhalf, &p.tmq2[c.s], &ctl->q_full, h * 64, y, zq);
     }
-    if (!mbar_wait(&ctl->k_empty[stage], phase ^ 1, p.wait_ns)) { fail(ctl, p.err); break; }
-    mbar_arrive_expect_tx(&ctl->k_full[stage], kTileBytes);
+    last_q_pc = pc;
+    ++pc;
     const int zk = (p.layer0 + c.l) * p.G + c.g;
-    for (int h = 0; h < 2; ++h)
-      tma_load_3d_hint(sK + stage * kTileBytes + h * kHalfBytes, &p.tmk[c.s], &ctl->k_full[stage],
-                       h * 64, c.j * kTileKeys, zk, pol_k);
-    last_ph[stage] = phase;
-    if (++stage == p.kstages) {
-      stage = 0;
-      phase ^= 1;
+    for (int j = c.j0; j < c.j0 + c.n; ++j) {
+      if (ctl->abort) break;
+      if (!mbar_wait(&ctl->k_empty[stage], phase ^ 1, p.wait_ns)) { fail(ctl, p.err); break; }
+      mbar_arrive_expect_tx(&ctl->k_full[stage], kTileBytes);
+      for (int h = 0; h < 2; ++h)
+        tma_load_3d_hint(sK + stage * kTileBytes + h * kHalfBytes, &p.tmk[c.s], &ctl->k_full[stage],
+                         h * 64, j * kTileKeys, zk, pol_k);
+      last_ph[stage] = phase;
+      if (++stage == p.kstages) {
+        stage = 0;
+        phase ^= 1;
+      }
     }
   }
   if (ctl->abort) {
@@ -239,19 +240,18 @@ __device__ void mma_loop(const ScoreParams& p, SmemCtl* ctl, const uint8_t* sQ, 
   // K stage and phase of tile jt = who, who + 2, ...
   int stage = who % p.kstages, phase = 0, pc = 0, own = 0;
   const uint32_t d0 = tmem + who * 256;
-  int64_t jt = 0;
-  TileIter c;
-  for (c.init(p, fb, fe); c.valid(); c.next(p), ++jt) {
-    if (ctl->abort) break;
-    if (c.first(fb)) {
-      if (!mbar_wait(&ctl->q_full, pc & 1, p.wait_ns)) { fail(ctl, p.err); break; }
-      if (PASS == 2) {
-        if (!mbar_wait(&ctl->x_full[pc & 1], (pc >> 1) & 1, p.wait_ns)) { fail(ctl, p.err); break; }
-        dbx = dbx0 + static_cast<uint64_t>((pc & 1) * ((p.q_rows * kXRowBytes) >> 4));
-      }
-      ++pc;
+  int jt = 0;
+  for (PieceIter c(p, fb, fe); c.valid() && !ctl->abort; c.next(p)) {
+    if (!mbar_wait(&ctl->q_full, pc & 1, p.wait_ns)) { fail(ctl, p.err); break; }
+    if (PASS == 2) {
+      if (!mbar_wait(&ctl->x_full[pc & 1], (pc >> 1) & 1, p.wait_ns)) { fail(ctl, p.err); break; }
+      dbx = dbx0 + static_cast<uint64_t>((pc & 1) * ((p.q_rows * kXRowBytes) >> 4));
     }
-    if ((jt & 1) == who) {
+    ++pc;
+    const int jt1 = jt + c.n;
+    // this issuer's tiles of the piece: those of its parity in the CTA's range
+    for (jt += (jt ^ who) & 1; jt < jt1; jt += 2) {
+      if (ctl->abort) break;
       if (!mbar_wait(&ctl->k_full[stage], phase, p.wait_ns)) { fail(ctl, p.err); break; }
       if (!mbar_wait(&ctl->t_empty[who], (own & 1) ^ 1, p.wait_ns)) { fail(ctl, p.err); break; }
       tc_fence_after();
@@ -290,7 +290,8 @@ __device__ void mma_loop(const ScoreParams& p, SmemCtl* ctl, const uint8_t* sQ, 
         phase ^= 1;
       }
     }
-    if (c.last()) mma_commit(&ctl->q_empty);
+    jt = jt1;
+    mma_commit(&ctl->q_empty);
   }
   // every MMA issued above must be complete before TMEM is released
   mma_commit(&ctl->drain);
@@ -411,34 +412,37 @@ __device__ __forceinline__ void lse_tile_slow(uint32_t base, int n, int lim, flo
 }
 
 // One row's running (reference m, sum s of exp2(z sc - m)) over this thread's
-// `nch` 16-key chunks of one tile, `lim` of which keys are valid.  The
+// NCH 16-key chunks of one tile, `lim` of which keys are valid.  The
 // reference is set on a piece's first tile and moves only when a tile's sum
 // exceeds 2^64 (a logit more than 64 above it, or overflow); that tile is then
 // redone.  Terms far below the reference underflow to zero, below the fp32
 // resolution of the sum.  A lane that is not `live` (a row past the group's
 // window rows) takes part in the warp-collective loads only.  The full-tile
 // path is straight-line; everything else goes through the slow path.
-__device__ __forceinline__ void lse_tile(uint32_t base, int nch, int lim, float sc, bool live, float& m, float& s) {
+template <int NCH>
+__device__ __forceinline__ void lse_tile(uint32_t base, int lim, float sc, bool live, float& m, float& s) {
   if (lim <= 0) return;   // lim is the same in every lane
-  if (lim < nch * 16 || __any_sync(kFull, m == -INFINITY)) {
-    lse_tile_slow(base, min(nch, (lim + 15) >> 4), lim, sc, live, m, s);
+  if (lim < NCH * 16 || __any_sync(kFull, m == -INFINITY)) {
+    lse_tile_slow(base, min(NCH, (lim + 15) >> 4), lim, sc, live, m, s);
     return;
   }
   const float2 sc2 = make_float2(sc, sc), nm2 = make_float2(-m, -m);
   float2 a0 = make_float2(0.f, 0.f), a1 = make_float2(0.f, 0.f);
-  stream16(base, nch, [&](const uint32_t(&r)[16], int) { exp2_acc16(r, sc2, nm2, a0, a1); });
+  stream16(base, NCH, [&](const uint32_t(&r)[16], int) { exp2_acc16(r, sc2, nm2, a0, a1); });
   const float2 a = fadd2(a0, a1);
   const float cs = a.x + a.y;
   if (__all_sync(kFull, !live || cs < 1.8446744e19f)) {   // below 2^64: the common case
     if (live) s += cs;
   } else {
-    lse_tile_slow(base, nch, lim, sc, live, m, s);
+    lse_tile_slow(base, NCH, lim, sc, live, m, s);
   }
 }
 
 }  // namespace
 
 // 20 warps share the register file: at most 96 registers a thread.
+// TWO: the group's window rows fill two M tiles (more than 128 rows).
+template <bool TWO>
 __global__ void __launch_bounds__(kScoreThreads, 1) k_score_lse(const __grid_constant__ ScoreParams p) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = align1024(smem_raw);
@@ -474,10 +478,9 @@ __global__ void __launch_bounds__(kScoreThreads, 1) k_score_lse(const __grid_con
     const int q = quad * 32 + lane;         // TMEM lane
     // two M tiles: warpgroup (mt, half) owns 64 keys of M tile mt;
     // one M tile: the four warpgroups own 32 keys each
-    const bool two = p.n_mtiles == 2;
-    const int mt = two ? (wg >> 1) : 0;
-    const int kofs = two ? (wg & 1) * 64 : wg * 32;
-    const int nch = two ? 4 : 2;
+    constexpr int NCH = TWO ? 4 : 2;         // 16-key chunks of a warp's tile
+    const int mt = TWO ? (wg >> 1) : 0;
+    const int kofs = TWO ? (wg & 1) * 64 : wg * 32;
     const int r = mt * kTileKeys + q;       // window row within the group
     const bool active = mt * kTileKeys + quad * 32 < p.rows;
     const uint32_t base0 = tmem + (static_cast<uint32_t>(quad * 32) << 16) + mt * kTileKeys + kofs;
@@ -485,51 +488,44 @@ __global__ void __launch_bounds__(kScoreThreads, 1) k_score_lse(const __grid_con
     float m = -INFINITY, s = 0.f;
     int jt = 0;
     bool dead = false;
-    int64_t piece_start = 0;
     // Every epilogue warp walks every tile and meets the piece-end barrier in
     // the same order; a warp whose wait ran out keeps walking without waiting.
-    TileIter c;
-    for (c.init(p, fb, fe); c.valid(); c.next(p)) {
-      const bool last = c.last();
-      if (c.first(fb)) {
-        piece_start = c.f;
-        m = -INFINITY;
-        s = 0.f;
-      }
-      const int ts = jt & 1;
-      if (!dead) {
+    for (PieceIter c(p, fb, fe); c.valid(); c.next(p)) {
+      m = -INFINITY;
+      s = 0.f;
+      int lim = p.seq[c.s].Lp - (c.j0 * kTileKeys + kofs);   // valid keys from this warp's first on
+      for (const int jt1 = jt + c.n; jt < jt1; ++jt, lim -= kTileKeys) {
+        if (dead) continue;
+        const int ts = jt & 1;
         if (!__all_sync(kFull, mbar_wait(&ctl->t_full[ts][mt], (jt >> 1) & 1, p.wait_ns))) {
           fail(ctl, p.err);
           dead = true;
-        } else {
-          tc_fence_after();
-          if (active) lse_tile(base0 + ts * 256, nch, p.seq[c.s].Lp - (c.j * kTileKeys + kofs), sc, r < p.rows, m, s);
-          tc_fence_before();
-          __syncwarp();
-          if (lane == 0) mbar_arrive(&ctl->t_empty[ts]);
+          continue;
         }
+        tc_fence_after();
+        if (active) lse_tile<NCH>(base0 + ts * 256, lim, sc, r < p.rows, m, s);
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&ctl->t_empty[ts]);
       }
-      if (last) {
-        // merge the key parts of each row, write the piece's partial
-        pbuf[wg * 128 + q] = make_float2(m, s);
-        named_bar_sync(1, kEpiThreads);
-        const bool writer = two ? (wg & 1) == 0 : wg == 0;
-        if (writer && r < p.rows && !dead) {
-          const int n = two ? 2 : 4;
-          const int w0 = two ? wg : 0;
-          float mx = -INFINITY;
-          for (int i = 0; i < n; ++i) mx = fmaxf(mx, pbuf[(w0 + i) * 128 + q].x);
-          float sum = 0.f;
-          if (mx != -INFINITY)
-            for (int i = 0; i < n; ++i) {
-              const float2 v = pbuf[(w0 + i) * 128 + q];
-              if (v.x != -INFINITY) sum += v.y * ex2_approx(v.x - mx);
-            }
-          p.partials[piece_start * kMaxRows + r] = make_float2(mx, sum);
-        }
-        named_bar_sync(1, kEpiThreads);   // pbuf is reused by the next piece
+      // merge the key parts of each row, write the piece's partial
+      pbuf[wg * 128 + q] = make_float2(m, s);
+      named_bar_sync(1, kEpiThreads);
+      const bool writer = TWO ? (wg & 1) == 0 : wg == 0;
+      if (writer && r < p.rows && !dead) {
+        constexpr int n = TWO ? 2 : 4;
+        const int w0 = TWO ? wg : 0;
+        float mx = -INFINITY;
+        for (int i = 0; i < n; ++i) mx = fmaxf(mx, pbuf[(w0 + i) * 128 + q].x);
+        float sum = 0.f;
+        if (mx != -INFINITY)
+          for (int i = 0; i < n; ++i) {
+            const float2 v = pbuf[(w0 + i) * 128 + q];
+            if (v.x != -INFINITY) sum += v.y * ex2_approx(v.x - mx);
+          }
+        p.partials[c.f * kMaxRows + r] = make_float2(mx, sum);
       }
-      ++jt;
+      named_bar_sync(1, kEpiThreads);   // pbuf is reused by the next piece
     }
   }
   __syncthreads();
@@ -581,18 +577,17 @@ __global__ void __launch_bounds__(kScoreThreads, 1) k_score_accum(const __grid_c
     const int nch = (nc >> 2) + (wg < (nc & 3) ? 1 : 0);
     const uint32_t base0 = tmem + (static_cast<uint32_t>(quad * 32) << 16) + ch0 * 16;
     const float sc = p.scale2, isc = 1.f / p.scale2, sqd = sqrtf(static_cast<float>(kHeadDim));
-    // the -lse operand of the piece `it` (whose row starts at flat tile r0),
-    // into buffer `buf`: window row et holds x = -lse2 / scale (= -lse sqrt(d)
+    // the -lse operand of the piece `it` into buffer `buf`: window row et holds x = -lse2 / scale (= -lse sqrt(d)
     // for a supplied natural-log normaliser) as three bf16 parts (x = hi + mid
     // + lo to about 2^-24 relative) in its K columns 0..2; rows past the
     // group's window rows get a large negative x (exp2 -> 0)
-    auto write_x = [&](const TileIter& it, int64_t r0, int buf) {
+    auto write_x = [&](const PieceIter& it, int buf) {
       if (et < p.n2) {
         float x = -3.0e38f;
         if (et < p.rows) {
           const float* lse = p.seq[it.s].lse;
           x = lse ? -lse[(static_cast<int64_t>(p.layer0 + it.l) * p.G + it.g) * p.rows + et] * sqd
-                  : -combine_lse2(p, r0, it.nt, et) * isc;
+                  : -combine_lse2(p, it.f - it.j0, it.nt, et) * isc;
         }
         const __nv_bfloat16 hi = __float2bfloat16_rn(x);
         const float r1 = x - __bfloat162float(hi);
@@ -610,8 +605,6 @@ __global__ void __launch_bounds__(kScoreThreads, 1) k_score_accum(const __grid_c
     };
     int jt = 0, kp = 0;
     bool dead = false;
-    float* dst = nullptr;   // the piece's unpooled row, at this thread's key of tile 0
-    int lp = 0;
     // The four column quarters of a key lie in four warps.  Each writes its
     // sum of tile j to slot j mod 8 before it releases the tile's accumulator
     // stage, so that a warp that finds tile j + 2 ready (the stage's next
@@ -626,55 +619,48 @@ __global__ void __launch_bounds__(kScoreThreads, 1) k_score_accum(const __grid_c
       const float* v = sS + (j & (kSumSlots - 1)) * (4 * kTileKeys) + q;
       *to = ((v[0] + v[kTileKeys]) + v[2 * kTileKeys]) + v[3 * kTileKeys];
     };
-    TileIter c;
-    c.init(p, fb, fe);
+    PieceIter c(p, fb, fe);
     if (c.valid()) {
       // the ones operand: bf16 1.0 in K columns 0..2 of core matrix 0, zeros elsewhere
       if (et < 16) {
         *reinterpret_cast<uint4*>(sX + et * 16) =
             et < 8 ? make_uint4(0x3F803F80u, 0x00003F80u, 0u, 0u) : make_uint4(0u, 0u, 0u, 0u);
       }
-      write_x(c, c.f - c.j, 0);
+      write_x(c, 0);
     }
     const float2 sc2 = make_float2(sc, sc), zero2 = make_float2(0.f, 0.f);
-    for (; c.valid(); c.next(p)) {
-      if (c.first(fb)) {
-        // the next piece's operand goes to the other buffer now, one piece
-        // ahead of its MMAs (this piece's buffer was written one piece earlier;
-        // the other one's readers, the previous piece's MMAs, are done)
-        const int64_t fn = c.f + (c.nt - c.j);
-        if (fn < fe) {
-          TileIter n;
-          n.init(p, fn, fe);
-          write_x(n, fn, (kp + 1) & 1);
-        }
-        ++kp;
-        const ScoreSeq& sq = p.seq[c.s];
-        lp = sq.Lp;
-        dst = sq.s_raw + static_cast<int64_t>(c.l * p.G + c.g) * raw_stride(lp) + q;
-      }
-      const int ts = jt & 1;
-      if (!dead) {
+    for (; c.valid(); ++kp) {
+      // the next piece's operand goes to the other buffer now, one piece
+      // ahead of its MMAs (this piece's buffer was written one piece earlier;
+      // the other one's readers, the previous piece's MMAs, are done)
+      PieceIter nx = c;
+      nx.next(p);
+      if (nx.valid()) write_x(nx, (kp + 1) & 1);
+      const ScoreSeq& sq = p.seq[c.s];
+      int left = sq.Lp - (c.j0 * kTileKeys + q);   // > 0: this thread's key of the tile is past key
+      float* dst = sq.s_raw + static_cast<int64_t>(c.l * p.G + c.g) * raw_stride(sq.Lp) + c.j0 * kTileKeys + q;
+      for (const int jt1 = jt + c.n; jt < jt1; ++jt, left -= kTileKeys, dst += kTileKeys) {
+        if (dead) continue;
+        const int ts = jt & 1;
         if (!__all_sync(kFull, mbar_wait(&ctl->t_full[ts][0], (jt >> 1) & 1, p.wait_ns))) {
           fail(ctl, p.err);
           dead = true;
-        } else {
-          tc_fence_after();
-          float2 a0 = make_float2(0.f, 0.f), a1 = make_float2(0.f, 0.f);
-          if (nch > 0)
-            stream16(base0 + ts * 256, nch, [&](const uint32_t(&v)[16], int) { exp2_acc16(v, sc2, zero2, a0, a1); });
-          const float2 a = fadd2(a0, a1);
-          sS[((jt & (kSumSlots - 1)) * 4 + wg) * kTileKeys + q] = a.x + a.y;
-          tc_fence_before();
-          __syncwarp();
-          if (lane == 0) mbar_arrive(&ctl->t_empty[ts]);
-          if (jt >= 2) flush(jt - 2, pend2);
-          const int key0 = c.j * kTileKeys;
-          pend2 = pend1;
-          pend1 = key0 + q < lp ? dst + key0 : nullptr;
+          continue;
         }
+        tc_fence_after();
+        float2 a0 = make_float2(0.f, 0.f), a1 = make_float2(0.f, 0.f);
+        if (nch > 0)
+          stream16(base0 + ts * 256, nch, [&](const uint32_t(&v)[16], int) { exp2_acc16(v, sc2, zero2, a0, a1); });
+        const float2 a = fadd2(a0, a1);
+        sS[((jt & (kSumSlots - 1)) * 4 + wg) * kTileKeys + q] = a.x + a.y;
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&ctl->t_empty[ts]);
+        if (jt >= 2) flush(jt - 2, pend2);
+        pend2 = pend1;
+        pend1 = left > 0 ? dst : nullptr;
       }
-      ++jt;
+      c = nx;
     }
     named_bar_sync(1, kEpiThreads);   // every warp's last sums are written (all reach this, also after a timeout)
     if (!dead) {
@@ -730,7 +716,8 @@ int score_kstages(int q_rows) {
 
 cudaError_t score_configure() {
   const int bytes = static_cast<int>(kSmemLimit);
-  cudaError_t e = cudaFuncSetAttribute(k_score_lse, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  cudaError_t e = cudaFuncSetAttribute(k_score_lse<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_score_lse<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
   if (e != cudaSuccess) return e;
   return cudaFuncSetAttribute(k_score_accum, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
 }
@@ -759,7 +746,7 @@ cudaError_t launch_pdl(void (*kernel)(Args...), dim3 grid, dim3 block, size_t sm
 }  // namespace
 
 cudaError_t score_lse_launch(const ScoreParams& p, int grid, cudaStream_t stream) {
-  return launch_pdl(k_score_lse, dim3(grid), dim3(kScoreThreads), score_smem_bytes(p.q_rows, p.kstages), stream, p);
+  return launch_pdl(p.n_mtiles == 2 ? k_score_lse<true> : k_score_lse<false>, dim3(grid), dim3(kScoreThreads), score_smem_bytes(p.q_rows, p.kstages), stream, p);
 }
 
 cudaError_t score_accum_launch(const ScoreParams& p, int grid, cudaStream_t stream) {
