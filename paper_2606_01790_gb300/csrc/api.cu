@@ -1075,13 +1075,22 @@ extern "C" starkv_status starkv_score_layer_noalloc(starkv_state* st, int32_t la
   if (!st->noalloc_scratch)
     return set_error(STARKV_ERR_CUDA, "the static scratch is unavailable on device %d: %s", st->device,
                      st->noalloc_error.c_str());
-  WsPlan plan;
-  plan_ws(st, seqs, nseq, 1, false, false, &plan);
-  if (plan.total > kNoAllocScratchBytes)
+  // The limit counts the pass-1 partials and four unpooled rows per group (the
+  // kernels use one), so that the accepted batches do not depend on how pass 2
+  // splits its columns.
+  const size_t G = st->cfg.n_kv_heads;
+  size_t need = 0, tiles = 0;
+  for (int i = 0; i < nseq; ++i) {
+    const int lp = seqs[i].L - st->cfg.window;
+    tiles += G * tiles_of(lp);
+    need += align256(G * 4 * raw_stride(lp) * sizeof(float));
+  }
+  need = std::max<size_t>(need + align256(tiles * kMaxRows * sizeof(float2)), 256);
+  if (need > kNoAllocScratchBytes)
     return set_error(STARKV_ERR_UNSUPPORTED,
                      "this call needs %zu bytes of scratch; the static scratch holds %zu bytes: "
                      "split the batch or use starkv_score_layer with a workspace",
-                     plan.total, kNoAllocScratchBytes);
+                     need, kNoAllocScratchBytes);
   return run_stages(st, seqs, nseq, layer, 1, kScore | kPool, st->noalloc_scratch, kNoAllocScratchBytes,
                     static_cast<cudaStream_t>(stream));
 }
