@@ -151,41 +151,42 @@ __device__ __forceinline__ uint32_t bf16x2_to_f16x2(uint32_t w) {
   return pack_half2(__uint_as_float(w << 16), __uint_as_float(w & 0xFFFF0000u));
 }
 
-// Coordinates of consecutive flat units [f0, f1), advanced without divisions.
-struct UnitIter {
-  int s, l, g, j, nu;
-  int64_t f, fe;
-  __device__ void init(const AttnParams& p, int64_t f0, int64_t f1) {
-    f = f0;
-    fe = f1;
-    s = l = g = j = nu = 0;
-    if (f >= fe) return;
+// The pieces of a CTA's flat range [f0, f1), in order: a run of n units j0, j0 +
+// 1, ... of one (seq, layer, group) row.  One decode at the start, no
+// divisions after it, and only counters inside a piece.
+struct PieceIter {
+  int s, l, g, j0, n, nu;
+  int rem;   // units of the range from this piece on
+  __device__ __forceinline__ PieceIter(const AttnParams& p, int64_t f0, int64_t f1)
+      : s(0), l(0), g(0), j0(0), n(0), nu(0), rem(static_cast<int>(f1 - f0)) {
+    if (rem <= 0) return;
     while (s + 1 < p.nseq && p.seq[s + 1].unit_base <= f0) ++s;
     nu = p.seq[s].nu;
     const int64_t u = f0 - p.seq[s].unit_base;
     const int per_layer = p.G * nu;
     l = static_cast<int>(u / per_layer);
-    const int rem = static_cast<int>(u - static_cast<int64_t>(l) * per_layer);
-    g = rem / nu;
-    j = rem - g * nu;
+    const int r = static_cast<int>(u - static_cast<int64_t>(l) * per_layer);
+    g = r / nu;
+    j0 = r - g * nu;
+    n = min(rem, nu - j0);
   }
-  __device__ bool valid() const { return f < fe; }
-  __device__ bool first(int64_t fb) const { return f == fb || j == 0; }
-  __device__ bool last() const { return f + 1 == fe || j + 1 == nu; }
-  __device__ int row(const AttnParams& p) const { return (s * p.nlayers + l) * p.G + g; }
-  __device__ void next(const AttnParams& p) {
-    ++f;
-    if (f >= fe) return;
-    if (++j < nu) return;
-    j = 0;
-    if (++g < p.G) return;
-    g = 0;
-    if (++l < p.nlayers) return;
-    l = 0;
-    do {
-      ++s;
-    } while (s + 1 < p.nseq && p.seq[s].nu == 0);
-    nu = p.seq[s].nu;
+  __device__ __forceinline__ bool valid() const { return rem > 0; }
+  __device__ __forceinline__ int row(const AttnParams& p) const { return (s * p.nlayers + l) * p.G + g; }
+  __device__ __forceinline__ void next(const AttnParams& p) {
+    rem -= n;
+    j0 = 0;
+    if (rem <= 0) return;
+    if (++g == p.G) {
+      g = 0;
+      if (++l == p.nlayers) {
+        l = 0;
+        do {
+          ++s;
+        } while (s + 1 < p.nseq && p.seq[s].nu == 0);
+        nu = p.seq[s].nu;
+      }
+    }
+    n = min(rem, nu);
   }
 };
 
@@ -204,29 +205,29 @@ __device__ void k_loader(const AttnParams& p, AttnCtl* ctl, uint8_t* sQ, uint8_t
   int stage = 0, phase = 0, pc = 0, last_q_pc = -1;
   int last_ph[kStages];
   for (int i = 0; i < kStages; ++i) last_ph[i] = -1;
-  UnitIter c;
-  for (c.init(p, fb, fe); c.valid(); c.next(p)) {
-    if (ctl->abort) break;
-    if (c.first(fb)) {
-      if (!mbar_wait(&ctl->q_empty, (pc & 1) ^ 1, p.wait_ns)) { fail(ctl, p.err); break; }
-      const int zq = p.layer0 + c.l, y = c.g * p.rows;
-      mbar_arrive_expect_tx(&ctl->q_full, p.rows * 256);
-      for (int h = 0; h < 2; ++h) {
-        tma_load_3d(sQ + h * qhalf, &p.tmqa[c.s], &ctl->q_full, h * 64, y, zq);
-        if (p.rows > 128) tma_load_3d(sQ + h * qhalf + 128 * 128, &p.tmqb[c.s], &ctl->q_full, h * 64, y + 128, zq);
-      }
-      last_q_pc = pc;
-      ++pc;
+  for (PieceIter c(p, fb, fe); c.valid() && !ctl->abort; c.next(p)) {
+    if (!mbar_wait(&ctl->q_empty, (pc & 1) ^ 1, p.wait_ns)) { fail(ctl, p.err); break; }
+    const int zq = p.layer0 + c.l, yq = c.g * p.rows;
+    mbar_arrive_expect_tx(&ctl->q_full, p.rows * 256);
+    for (int h = 0; h < 2; ++h) {
+      tma_load_3d(sQ + h * qhalf, &p.tmqa[c.s], &ctl->q_full, h * 64, yq, zq);
+      if (p.rows > 128) tma_load_3d(sQ + h * qhalf + 128 * 128, &p.tmqb[c.s], &ctl->q_full, h * 64, yq + 128, zq);
     }
-    if (!mbar_wait(&ctl->k_empty[stage], phase ^ 1, p.wait_ns)) { fail(ctl, p.err); break; }
-    mbar_arrive_expect_tx(&ctl->k_full[stage], kUnitBytes);
-    const int zk = (p.layer0 + c.l) * p.G + c.g, y = c.j * kAttnUnitKeys;
-    for (int h = 0; h < 2; ++h)
-      tma_load_3d_hint(sK + stage * kUnitBytes + h * kHalfBytes, &p.tmk[c.s], &ctl->k_full[stage], h * 64, y, zk, pol);
-    last_ph[stage] = phase;
-    if (++stage == p.kv_stages) {
-      stage = 0;
-      phase ^= 1;
+    last_q_pc = pc;
+    ++pc;
+    const int zk = (p.layer0 + c.l) * p.G + c.g;
+    for (int j = c.j0; j < c.j0 + c.n; ++j) {
+      if (ctl->abort) break;
+      if (!mbar_wait(&ctl->k_empty[stage], phase ^ 1, p.wait_ns)) { fail(ctl, p.err); break; }
+      mbar_arrive_expect_tx(&ctl->k_full[stage], kUnitBytes);
+      for (int h = 0; h < 2; ++h)
+        tma_load_3d_hint(sK + stage * kUnitBytes + h * kHalfBytes, &p.tmk[c.s], &ctl->k_full[stage], h * 64,
+                         j * kAttnUnitKeys, zk, pol);
+      last_ph[stage] = phase;
+      if (++stage == p.kv_stages) {
+        stage = 0;
+        phase ^= 1;
+      }
     }
   }
   if (ctl->abort) {   // every issued copy completes before the CTA can exit
@@ -242,18 +243,20 @@ __device__ void v_loader(const AttnParams& p, AttnCtl* ctl, uint8_t* sV, int64_t
   int stage = 0, phase = 0;
   int last_ph[kStages];
   for (int i = 0; i < kStages; ++i) last_ph[i] = -1;
-  UnitIter c;
-  for (c.init(p, fb, fe); c.valid(); c.next(p)) {
-    if (ctl->abort) break;
-    if (!mbar_wait(&ctl->v_empty[stage], phase ^ 1, p.wait_ns)) { fail(ctl, p.err); break; }
-    mbar_arrive_expect_tx(&ctl->v_full[stage], kUnitBytes);
-    const int zk = (p.layer0 + c.l) * p.G + c.g, y = c.j * kAttnUnitKeys;
-    for (int h = 0; h < 2; ++h)
-      tma_load_3d_hint(sV + stage * kUnitBytes + h * kHalfBytes, &p.tmv[c.s], &ctl->v_full[stage], h * 64, y, zk, pol);
-    last_ph[stage] = phase;
-    if (++stage == p.kv_stages) {
-      stage = 0;
-      phase ^= 1;
+  for (PieceIter c(p, fb, fe); c.valid() && !ctl->abort; c.next(p)) {
+    const int zk = (p.layer0 + c.l) * p.G + c.g;
+    for (int j = c.j0; j < c.j0 + c.n; ++j) {
+      if (ctl->abort) break;
+      if (!mbar_wait(&ctl->v_empty[stage], phase ^ 1, p.wait_ns)) { fail(ctl, p.err); break; }
+      mbar_arrive_expect_tx(&ctl->v_full[stage], kUnitBytes);
+      for (int h = 0; h < 2; ++h)
+        tma_load_3d_hint(sV + stage * kUnitBytes + h * kHalfBytes, &p.tmv[c.s], &ctl->v_full[stage], h * 64,
+                         j * kAttnUnitKeys, zk, pol);
+      last_ph[stage] = phase;
+      if (++stage == p.kv_stages) {
+        stage = 0;
+        phase ^= 1;
+      }
     }
   }
   if (ctl->abort)
@@ -271,39 +274,39 @@ __device__ void mma_s_loop(const AttnParams& p, AttnCtl* ctl, const uint8_t* sQ,
   const uint64_t dq0 = sdesc_k_sw128(smem_u32(sQ));
   const uint32_t qhalf16 = (p.q_rows * 128) >> 4;
   int stage = 0, kphase = 0, pc = 0;
-  int64_t ui = 0;
-  UnitIter c;
-  for (c.init(p, fb, fe); c.valid(); c.next(p), ++ui) {
-    if (ctl->abort) break;
-    if (c.first(fb)) {
-      if (!mbar_wait(&ctl->q_full, pc & 1, p.wait_ns)) { fail(ctl, p.err); break; }
-      ++pc;
-    }
-    const int t = static_cast<int>(ui & 1);
-    if (!mbar_wait(&ctl->k_full[stage], kphase, p.wait_ns)) { fail(ctl, p.err); break; }
-    if (!mbar_wait(&ctl->s_empty[t], static_cast<uint32_t>(((ui >> 1) & 1) ^ 1), p.wait_ns)) { fail(ctl, p.err); break; }
-    tc_fence_after();
-    const uint64_t dk = sdesc_k_sw128(smem_u32(sK + stage * kUnitBytes));
+  uint32_t ui = 0;
+  const uint64_t dk0 = sdesc_k_sw128(smem_u32(sK));
+  for (PieceIter c(p, fb, fe); c.valid() && !ctl->abort; c.next(p)) {
+    if (!mbar_wait(&ctl->q_full, pc & 1, p.wait_ns)) { fail(ctl, p.err); break; }
+    ++pc;
+    for (int i = 0; i < c.n; ++i, ++ui) {
+      if (ctl->abort) break;
+      const int t = static_cast<int>(ui & 1);
+      if (!mbar_wait(&ctl->k_full[stage], kphase, p.wait_ns)) { fail(ctl, p.err); break; }
+      if (!mbar_wait(&ctl->s_empty[t], ((ui >> 1) & 1) ^ 1, p.wait_ns)) { fail(ctl, p.err); break; }
+      tc_fence_after();
+      const uint64_t dk = dk0 + static_cast<uint64_t>(stage * (kUnitBytes >> 4));
 #pragma unroll
-    for (int mt = 0; mt < 2; ++mt) {
-      if (mt >= p.n_mtiles) break;
-      // M tile 1 reads rows 128..255 of each Q half; rows past q_rows feed
-      // accumulator rows that no thread reads
-      const uint64_t dq = dq0 + static_cast<uint64_t>(mt * ((128 * 128) >> 4));
+      for (int mt = 0; mt < 2; ++mt) {
+        if (mt >= p.n_mtiles) break;
+        // M tile 1 reads rows 128..255 of each Q half; rows past q_rows feed
+        // accumulator rows that no thread reads
+        const uint64_t dq = dq0 + static_cast<uint64_t>(mt * ((128 * 128) >> 4));
 #pragma unroll
-      for (int kk = 0; kk < 8; ++kk) {
-        const uint32_t koff16 = (kk >> 2) * (kHalfBytes >> 4) + (kk & 3) * 2;
-        const uint32_t qoff16 = (kk >> 2) * qhalf16 + (kk & 3) * 2;
-        mma_bf16(tmem + 256 + t * 128 + mt * kAttnUnitKeys, dq + qoff16, dk + koff16, idesc_s, kk > 0);
+        for (int kk = 0; kk < 8; ++kk) {
+          const uint32_t koff16 = (kk >> 2) * (kHalfBytes >> 4) + (kk & 3) * 2;
+          const uint32_t qoff16 = (kk >> 2) * qhalf16 + (kk & 3) * 2;
+          mma_bf16(tmem + 256 + t * 128 + mt * kAttnUnitKeys, dq + qoff16, dk + koff16, idesc_s, kk > 0);
+        }
+        mma_commit(&ctl->s_full[t][mt]);   // that M tile's softmax starts without waiting for the next
       }
-      mma_commit(&ctl->s_full[t][mt]);   // that M tile's softmax starts without waiting for the next
+      mma_commit(&ctl->k_empty[stage]);
+      if (++stage == p.kv_stages) {
+        stage = 0;
+        kphase ^= 1;
+      }
     }
-    mma_commit(&ctl->k_empty[stage]);
-    if (c.last()) mma_commit(&ctl->q_empty);
-    if (++stage == p.kv_stages) {
-      stage = 0;
-      kphase ^= 1;
-    }
+    mma_commit(&ctl->q_empty);
   }
   // every MMA issued above must be complete before TMEM is released
   mma_commit(&ctl->drain);
@@ -314,39 +317,40 @@ __device__ void mma_pv_loop(const AttnParams& p, AttnCtl* ctl, const uint8_t* sV
                             int64_t fe) {
   const uint32_t idesc_o = idesc_f16_bmn(128, kHeadDim);
   int stage = 0, kphase = 0;
-  int64_t ui = 0;
-  UnitIter c;
-  for (c.init(p, fb, fe); c.valid(); c.next(p), ++ui) {
-    if (ctl->abort) break;
-    const int t = static_cast<int>(ui & 1);
-    if (!mbar_wait(&ctl->v_ready[stage], kphase, p.wait_ns)) { fail(ctl, p.err); break; }
-    const bool first = c.first(fb);   // the piece's first product overwrites O
-    const uint64_t dv = sdesc_mn_sw128(smem_u32(sV + stage * kUnitBytes), kHalfBytes, 1024);
-    bool ok = true;
+  uint32_t ui = 0;
+  const uint64_t dv0 = sdesc_mn_sw128(smem_u32(sV), kHalfBytes, 1024);
+  for (PieceIter c(p, fb, fe); c.valid() && !ctl->abort; c.next(p)) {
+    for (int i = 0; i < c.n; ++i, ++ui) {
+      if (ctl->abort) break;
+      const int t = static_cast<int>(ui & 1);
+      if (!mbar_wait(&ctl->v_ready[stage], kphase, p.wait_ns)) { fail(ctl, p.err); break; }
+      const uint64_t dv = dv0 + static_cast<uint64_t>(stage * (kUnitBytes >> 4));
+      bool ok = true;
 #pragma unroll
-    for (int mt = 0; mt < 2; ++mt) {
-      if (mt >= p.n_mtiles) break;
-      // each M tile's product as soon as its P is written
-      if (!mbar_wait(&ctl->p_full[t][mt], static_cast<uint32_t>((ui >> 1) & 1), p.wait_ns)) {
-        ok = false;
+      for (int mt = 0; mt < 2; ++mt) {
+        if (mt >= p.n_mtiles) break;
+        // each M tile's product as soon as its P is written
+        if (!mbar_wait(&ctl->p_full[t][mt], (ui >> 1) & 1, p.wait_ns)) {
+          ok = false;
+          break;
+        }
+        tc_fence_after();
+        const uint32_t ap = tmem + 256 + t * 128 + mt * kAttnUnitKeys;   // P of M tile mt over its S columns
+#pragma unroll
+        for (int kk = 0; kk < 4; ++kk)   // 16 keys per step: +8 columns of P, +16 rows of V; the piece's first product overwrites O
+          mma_f16_ts(tmem + mt * kHeadDim, ap + kk * 8, dv + static_cast<uint64_t>(kk * 128), idesc_o,
+                     (i > 0 || kk > 0) ? 1u : 0u);
+      }
+      if (!ok) {
+        fail(ctl, p.err);
         break;
       }
-      tc_fence_after();
-      const uint32_t ap = tmem + 256 + t * 128 + mt * kAttnUnitKeys;   // P of M tile mt over its S columns
-#pragma unroll
-      for (int kk = 0; kk < 4; ++kk)   // 16 keys per step: +8 columns of P, +16 rows of V
-        mma_f16_ts(tmem + mt * kHeadDim, ap + kk * 8, dv + static_cast<uint64_t>(kk * 128), idesc_o,
-                   (!first || kk > 0) ? 1u : 0u);
-    }
-    if (!ok) {
-      fail(ctl, p.err);
-      break;
-    }
-    mma_commit(&ctl->v_empty[stage]);
-    mma_commit(&ctl->s_empty[t]);   // S stage t (holding P) is free for S two units later
-    if (++stage == p.kv_stages) {
-      stage = 0;
-      kphase ^= 1;
+      mma_commit(&ctl->v_empty[stage]);
+      mma_commit(&ctl->s_empty[t]);   // S stage t (holding P) is free for S two units later
+      if (++stage == p.kv_stages) {
+        stage = 0;
+        kphase ^= 1;
+      }
     }
   }
   mma_commit(&ctl->drain);
@@ -366,40 +370,42 @@ __device__ __forceinline__ float unit_max(const uint32_t (&z)[4][16], int lim) {
   return fmaxf(fmaxf(fmaxf(pm[0], pm[1]), fmaxf(pm[2], pm[3])), fmaxf(fmaxf(pm[4], pm[5]), fmaxf(pm[6], pm[7])));
 }
 
-// exp2 and pack of one 16-key chunk (keys k0 .. k0 + 15)
-__device__ __forceinline__ void exp_pack_chunk(const uint32_t (&z)[16], int k0, int lim, bool live, float2 sc2,
-                                               float2 nm2, float2 (&acc)[4], uint32_t (&h)[8]) {
+// exp2 and pack of one 16-key chunk (keys k0 .. k0 + 15).  FULL: every key of
+// the unit is valid, so that nothing is compared or selected per element (a row
+// that is not live then holds garbage, which only its own O row ever sees and
+// nothing reads).
+template <bool FULL>
+__device__ __forceinline__ void exp_pack_chunk(const uint32_t (&z)[16], int k0, int lim, float2 sc2, float2 nm2,
+                                               float2 (&acc)[4], uint32_t (&h)[8]) {
 #pragma unroll
   for (int i = 0; i < 16; i += 2) {
     const float2 e = ffma2(make_float2(__uint_as_float(z[i]), __uint_as_float(z[i + 1])), sc2, nm2);
     const int k = k0 + i;
-    const float p0 = (live && k < lim) ? ex2_approx(e.x) : 0.f;
-    const float p1 = (live && k + 1 < lim) ? ex2_approx(e.y) : 0.f;
+    const float p0 = (FULL || k < lim) ? ex2_approx(e.x) : 0.f;
+    const float p1 = (FULL || k + 1 < lim) ? ex2_approx(e.y) : 0.f;
     acc[(i >> 1) & 3] = fadd2(acc[(i >> 1) & 3], make_float2(p0, p1));
     h[i >> 1] = pack_half2(p0, p1);
   }
 }
 
-// p = exp2(z c2 - m) of the unit's 64 keys (0 past `lim` and in a row that
-// is not live) as fp16 pairs h[q][j] = (p[16 q + 2 j], p[16 q + 2 j + 1]), the
+// p = exp2(z c2 - m) of the unit's 64 keys (0 past `lim`) as fp16 pairs h[q][j] = (p[16 q + 2 j], p[16 q + 2 j + 1]), the
 // lower key in the low half; returns the sum of the p.
-__device__ __forceinline__ float exp_pack_p(const uint32_t (&z)[4][16], int lim, bool live, float c2, float m,
+__device__ __forceinline__ float exp_pack_p(const uint32_t (&z)[4][16], int lim, float c2, float m,
                                             uint32_t (&h)[4][8]) {
   const float2 sc2 = make_float2(c2, c2), nm2 = make_float2(-m, -m);
   float2 acc[4] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f),
                    make_float2(0.f, 0.f)};   // four independent running sums
 #pragma unroll
-  for (int q = 0; q < 4; ++q) exp_pack_chunk(z[q], 16 * q, lim, live, sc2, nm2, acc, h[q]);
+  for (int q = 0; q < 4; ++q) exp_pack_chunk<false>(z[q], 16 * q, lim, sc2, nm2, acc, h[q]);
   const float2 a01 = fadd2(acc[0], acc[1]), a23 = fadd2(acc[2], acc[3]);
   const float2 a = fadd2(a01, a23);
   return a.x + a.y;
 }
 
-// exp_pack_p reading S itself from `scol` in two halves, the second half's
+// exp_pack_p of a unit of 64 valid keys, reading S itself from `scol` in two halves, the second half's
 // loads in flight under the first half's arithmetic (measured faster than
 // waiting for all four loads first, and than one 16-column load ahead)
-__device__ __forceinline__ float exp_pack_p_streamed(uint32_t scol, int lim, bool live, float c2, float m,
-                                                     uint32_t (&h)[4][8]) {
+__device__ __forceinline__ float exp_pack_p_streamed(uint32_t scol, float c2, float m, uint32_t (&h)[4][8]) {
   const float2 sc2 = make_float2(c2, c2), nm2 = make_float2(-m, -m);
   float2 acc[4] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f),
                    make_float2(0.f, 0.f)};   // four independent running sums
@@ -410,12 +416,12 @@ __device__ __forceinline__ float exp_pack_p_streamed(uint32_t scol, int lim, boo
   tmem_wait16(a1);
   tmem_ld16_async(scol + 32, b0);
   tmem_ld16_async(scol + 48, b1);
-  exp_pack_chunk(a0, 0, lim, live, sc2, nm2, acc, h[0]);
-  exp_pack_chunk(a1, 16, lim, live, sc2, nm2, acc, h[1]);
+  exp_pack_chunk<true>(a0, 0, kAttnUnitKeys, sc2, nm2, acc, h[0]);
+  exp_pack_chunk<true>(a1, 16, kAttnUnitKeys, sc2, nm2, acc, h[1]);
   tmem_wait16(b0);
   tmem_wait16(b1);
-  exp_pack_chunk(b0, 32, lim, live, sc2, nm2, acc, h[2]);
-  exp_pack_chunk(b1, 48, lim, live, sc2, nm2, acc, h[3]);
+  exp_pack_chunk<true>(b0, 32, kAttnUnitKeys, sc2, nm2, acc, h[2]);
+  exp_pack_chunk<true>(b1, 48, kAttnUnitKeys, sc2, nm2, acc, h[3]);
   const float2 a01 = fadd2(acc[0], acc[1]), a23 = fadd2(acc[2], acc[3]);
   const float2 a = fadd2(a01, a23);
   return a.x + a.y;
@@ -464,12 +470,12 @@ __device__ __forceinline__ bool softmax_unit(const AttnParams& p, bool wactive, 
   uint32_t z[4][16];
   uint32_t h[4][8];
   float us;
-  if (fresh) {
+  if (fresh || lim < kAttnUnitKeys) {
     load_s(scol, z);
-    m = unit_max(z, lim) * c2;
-    us = exp_pack_p(z, lim, live, c2, m, h);
+    if (fresh) m = unit_max(z, lim) * c2;
+    us = exp_pack_p(z, lim, c2, m, h);
   } else {
-    us = exp_pack_p_streamed(scol, lim, live, c2, m, h);
+    us = exp_pack_p_streamed(scol, c2, m, h);
   }
   if (__any_sync(kFull, live && us > 32768.f)) {   // rare
     load_s(scol, z);   // z again, so that it need not live across the first pass
@@ -485,7 +491,7 @@ __device__ __forceinline__ bool softmax_unit(const AttnParams& p, bool wactive, 
     }
     // P again in every lane (the same values where the reference stayed), so
     // that the first h need not live across the reload either
-    us = exp_pack_p(z, lim, live, c2, m, h);
+    us = exp_pack_p(z, lim, c2, m, h);
   }
 #pragma unroll
   for (int q = 0; q < 4; ++q) tmem_st8(scol + q * 8, h[q]);   // keys 16 q ..: columns 8 q ..
@@ -510,56 +516,56 @@ __device__ void softmax_loop(const AttnParams& p, AttnCtl* ctl, uint32_t tmem, i
   const uint32_t lane_base = tmem + (static_cast<uint32_t>(quad * 32) << 16);
   float m = -INFINITY, l = 0.f;
   uint32_t ui = 0;
-  UnitIter c;
-  for (c.init(p, fb, fe); c.valid(); c.next(p), ++ui) {
-    if (ctl->abort) break;
-    const bool first = c.first(fb), last = c.last();
-    const int t = static_cast<int>(ui % kSStages);
-    const uint32_t par = (ui / kSStages) & 1u;
-    const uint32_t scol = s_col0 + t * s_stride;   // this unit's S, then P, columns
-    if (!__all_sync(kFull, mbar_wait(&ctl->s_full[t][mt], par, p.wait_ns))) {
-      fail(ctl, p.err);
-      break;
-    }
-    tc_fence_after();
-    const int lim = p.seq[c.s].Lp - c.j * kAttnUnitKeys;   // valid keys of the unit (>= 1)
-    const uint32_t up = ui - 1;   // the previous unit (a piece's first unit never moves)
-    if (!softmax_unit(p, wactive, live, first, lim, lane_base + scol, lane_base + o_col,
-                      &ctl->s_empty[up % kSStages], (up / kSStages) & 1u, m, l)) {
-      fail(ctl, p.err);
-      break;
-    }
-    tmem_wait_st();
-    tc_fence_before();
-    __syncwarp();
-    if (lane == 0) mbar_arrive(&ctl->p_full[t][mt]);
-    if (last) {
-      // the piece's partial: (m, l) and the unnormalised O rows, once the
-      // product of this last unit is done
-      if (!__all_sync(kFull, mbar_wait(&ctl->s_empty[t], par, p.wait_ns))) {
+  for (PieceIter c(p, fb, fe); c.valid() && !ctl->abort; c.next(p)) {
+    int lim = p.seq[c.s].Lp - c.j0 * kAttnUnitKeys;   // valid keys from the unit's first on (>= 1)
+    for (int i = 0; i < c.n; ++i, ++ui, lim -= kAttnUnitKeys) {
+      if (ctl->abort) break;
+      const int t = static_cast<int>(ui % kSStages);
+      const uint32_t par = (ui / kSStages) & 1u;
+      const uint32_t scol = s_col0 + t * s_stride;   // this unit's S, then P, columns
+      if (!__all_sync(kFull, mbar_wait(&ctl->s_full[t][mt], par, p.wait_ns))) {
         fail(ctl, p.err);
         break;
       }
       tc_fence_after();
-      const int64_t slot = static_cast<int64_t>(c.row(p)) + slot0;
-      if (wactive) {
-        float* dst = p.part_o + (slot * kMaxRows + r) * kHeadDim;
-#pragma unroll 1
-        for (int ch = 0; ch < kHeadDim / 16; ++ch) {
-          uint32_t o[16];
-          tmem_ld16_async(lane_base + o_col + ch * 16, o);
-          tmem_wait16(o);
-          if (live)
-#pragma unroll
-            for (int i = 0; i < 16; i += 4)
-              *reinterpret_cast<float4*>(dst + ch * 16 + i) =
-                  make_float4(__uint_as_float(o[i]), __uint_as_float(o[i + 1]), __uint_as_float(o[i + 2]),
-                              __uint_as_float(o[i + 3]));
-        }
-        if (live) p.part_ml[slot * kMaxRows + r] = make_float2(m, l);
+      const uint32_t up = ui - 1;   // the previous unit (a piece's first unit never moves)
+      if (!softmax_unit(p, wactive, live, i == 0, lim, lane_base + scol, lane_base + o_col,
+                        &ctl->s_empty[up % kSStages], (up / kSStages) & 1u, m, l)) {
+        fail(ctl, p.err);
+        break;
       }
+      tmem_wait_st();
       tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&ctl->p_full[t][mt]);
     }
+    if (ctl->abort) break;
+    // the piece's partial: (m, l) and the unnormalised O rows, once the
+    // product of its last unit is done
+    const uint32_t lu = ui - 1;
+    if (!__all_sync(kFull, mbar_wait(&ctl->s_empty[lu % kSStages], (lu / kSStages) & 1u, p.wait_ns))) {
+      fail(ctl, p.err);
+      break;
+    }
+    tc_fence_after();
+    const int64_t slot = static_cast<int64_t>(c.row(p)) + slot0;
+    if (wactive) {
+      float* dst = p.part_o + (slot * kMaxRows + r) * kHeadDim;
+#pragma unroll 1
+      for (int ch = 0; ch < kHeadDim / 16; ++ch) {
+        uint32_t o[16];
+        tmem_ld16_async(lane_base + o_col + ch * 16, o);
+        tmem_wait16(o);
+        if (live)
+#pragma unroll
+          for (int i = 0; i < 16; i += 4)
+            *reinterpret_cast<float4*>(dst + ch * 16 + i) =
+                make_float4(__uint_as_float(o[i]), __uint_as_float(o[i + 1]), __uint_as_float(o[i + 2]),
+                            __uint_as_float(o[i + 3]));
+      }
+      if (live) p.part_ml[slot * kMaxRows + r] = make_float2(m, l);
+    }
+    tc_fence_before();
   }
 }
 
@@ -569,7 +575,7 @@ template <int NW>
 __device__ void convert_loop(const AttnParams& p, AttnCtl* ctl, uint8_t* sV, int kv_stages, int ct, int lane, int64_t fb,
                              int64_t fe) {
   int stage = 0, phase = 0;
-  for (int64_t f = fb; f < fe; ++f) {
+  for (int n = static_cast<int>(fe - fb); n > 0; --n) {
     if (ctl->abort) break;
     if (!__all_sync(kFull, mbar_wait(&ctl->v_full[stage], phase, p.wait_ns))) {
       fail(ctl, p.err);
