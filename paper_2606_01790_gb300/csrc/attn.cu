@@ -267,94 +267,102 @@ __device__ void v_loader(const AttnParams& p, AttnCtl* ctl, uint8_t* sV, int64_t
 // Two MMA issuers walk the same units: warp 1 issues S(u) into S stage u & 1
 // as soon as the stage is free and K(u) has landed, warp 2 issues
 // O += P(u) V(u) once the softmax has written P(u) and V(u) is fp16, so that
-// S of the next units runs ahead of the products.
+// S of the next units runs ahead of the products.  Each runs as a whole warp
+// (elect_one).
 __device__ void mma_s_loop(const AttnParams& p, AttnCtl* ctl, const uint8_t* sQ, const uint8_t* sK, uint32_t tmem,
                            int64_t fb, int64_t fe) {
   const uint32_t idesc_s = idesc_bf16(128, kAttnUnitKeys);
-  const uint64_t dq0 = sdesc_k_sw128(smem_u32(sQ));
+  const uint64_t dq0 = sdesc_k_sw128(smem_u32(sQ)), dk0 = sdesc_k_sw128(smem_u32(sK));
   const uint32_t qhalf16 = (p.q_rows * 128) >> 4;
   int stage = 0, kphase = 0, pc = 0;
   uint32_t ui = 0;
-  const uint64_t dk0 = sdesc_k_sw128(smem_u32(sK));
-  for (PieceIter c(p, fb, fe); c.valid() && !ctl->abort; c.next(p)) {
-    if (!mbar_wait(&ctl->q_full, pc & 1, p.wait_ns)) { fail(ctl, p.err); break; }
+  bool ok = true;
+  for (PieceIter c(p, fb, fe); ok && c.valid(); c.next(p)) {
+    ok = !__any_sync(kFull, ctl->abort) && warp_wait(&ctl->q_full, pc & 1, p.wait_ns);
     ++pc;
-    for (int i = 0; i < c.n; ++i, ++ui) {
-      if (ctl->abort) break;
+    for (int i = 0; ok && i < c.n; ++i, ++ui) {
       const int t = static_cast<int>(ui & 1);
-      if (!mbar_wait(&ctl->k_full[stage], kphase, p.wait_ns)) { fail(ctl, p.err); break; }
-      if (!mbar_wait(&ctl->s_empty[t], ((ui >> 1) & 1) ^ 1, p.wait_ns)) { fail(ctl, p.err); break; }
+      ok = warp_wait(&ctl->k_full[stage], kphase, p.wait_ns) &&
+           warp_wait(&ctl->s_empty[t], ((ui >> 1) & 1) ^ 1, p.wait_ns);
+      if (!ok) break;
       tc_fence_after();
       const uint64_t dk = dk0 + static_cast<uint64_t>(stage * (kUnitBytes >> 4));
+      if (elect_one()) {
 #pragma unroll
-      for (int mt = 0; mt < 2; ++mt) {
-        if (mt >= p.n_mtiles) break;
-        // M tile 1 reads rows 128..255 of each Q half; rows past q_rows feed
-        // accumulator rows that no thread reads
-        const uint64_t dq = dq0 + static_cast<uint64_t>(mt * ((128 * 128) >> 4));
+        for (int mt = 0; mt < 2; ++mt) {
+          if (mt >= p.n_mtiles) break;
+          // M tile 1 reads rows 128..255 of each Q half; rows past q_rows feed
+          // accumulator rows that no thread reads
+          const uint64_t dq = dq0 + static_cast<uint64_t>(mt * ((128 * 128) >> 4));
 #pragma unroll
-        for (int kk = 0; kk < 8; ++kk) {
-          const uint32_t koff16 = (kk >> 2) * (kHalfBytes >> 4) + (kk & 3) * 2;
-          const uint32_t qoff16 = (kk >> 2) * qhalf16 + (kk & 3) * 2;
-          mma_bf16(tmem + 256 + t * 128 + mt * kAttnUnitKeys, dq + qoff16, dk + koff16, idesc_s, kk > 0);
+          for (int kk = 0; kk < 8; ++kk) {
+            const uint32_t koff16 = (kk >> 2) * (kHalfBytes >> 4) + (kk & 3) * 2;
+            const uint32_t qoff16 = (kk >> 2) * qhalf16 + (kk & 3) * 2;
+            mma_bf16(tmem + 256 + t * 128 + mt * kAttnUnitKeys, dq + qoff16, dk + koff16, idesc_s, kk > 0);
+          }
+          mma_commit(&ctl->s_full[t][mt]);   // that M tile's softmax starts without waiting for the next
         }
-        mma_commit(&ctl->s_full[t][mt]);   // that M tile's softmax starts without waiting for the next
+        mma_commit(&ctl->k_empty[stage]);
+        if (i + 1 == c.n) mma_commit(&ctl->q_empty);
       }
-      mma_commit(&ctl->k_empty[stage]);
+      __syncwarp();
       if (++stage == p.kv_stages) {
         stage = 0;
         kphase ^= 1;
       }
     }
-    mma_commit(&ctl->q_empty);
   }
-  // every MMA issued above must be complete before TMEM is released
-  mma_commit(&ctl->drain);
-  mbar_wait(&ctl->drain, 0, drain_limit(p.wait_ns));
+  if (!ok) fail(ctl, p.err);
+  // every MMA issued above must be complete before TMEM is released (the
+  // commit tracks the electing lane's: elect_one picks the same lane each time)
+  if (elect_one()) mma_commit(&ctl->drain);
+  warp_wait(&ctl->drain, 0, drain_limit(p.wait_ns));
 }
 
 __device__ void mma_pv_loop(const AttnParams& p, AttnCtl* ctl, const uint8_t* sV, uint32_t tmem, int64_t fb,
                             int64_t fe) {
   const uint32_t idesc_o = idesc_f16_bmn(128, kHeadDim);
-  int stage = 0, kphase = 0;
-  uint32_t ui = 0;
   const uint64_t dv0 = sdesc_mn_sw128(smem_u32(sV), kHalfBytes, 1024);
-  for (PieceIter c(p, fb, fe); c.valid() && !ctl->abort; c.next(p)) {
-    for (int i = 0; i < c.n; ++i, ++ui) {
-      if (ctl->abort) break;
+  int stage = 0, vphase = 0;
+  uint32_t ui = 0;
+  bool ok = true;
+  for (PieceIter c(p, fb, fe); ok && c.valid(); c.next(p)) {
+    ok = !__any_sync(kFull, ctl->abort);
+    for (int i = 0; ok && i < c.n; ++i, ++ui) {
       const int t = static_cast<int>(ui & 1);
-      if (!mbar_wait(&ctl->v_ready[stage], kphase, p.wait_ns)) { fail(ctl, p.err); break; }
+      ok = warp_wait(&ctl->v_ready[stage], vphase, p.wait_ns);
       const uint64_t dv = dv0 + static_cast<uint64_t>(stage * (kUnitBytes >> 4));
-      bool ok = true;
 #pragma unroll
       for (int mt = 0; mt < 2; ++mt) {
-        if (mt >= p.n_mtiles) break;
+        if (mt >= p.n_mtiles || !ok) break;
         // each M tile's product as soon as its P is written
-        if (!mbar_wait(&ctl->p_full[t][mt], (ui >> 1) & 1, p.wait_ns)) {
-          ok = false;
-          break;
-        }
+        ok = warp_wait(&ctl->p_full[t][mt], (ui >> 1) & 1, p.wait_ns);
+        if (!ok) break;
         tc_fence_after();
         const uint32_t ap = tmem + 256 + t * 128 + mt * kAttnUnitKeys;   // P of M tile mt over its S columns
+        if (elect_one()) {
 #pragma unroll
-        for (int kk = 0; kk < 4; ++kk)   // 16 keys per step: +8 columns of P, +16 rows of V; the piece's first product overwrites O
-          mma_f16_ts(tmem + mt * kHeadDim, ap + kk * 8, dv + static_cast<uint64_t>(kk * 128), idesc_o,
-                     (i > 0 || kk > 0) ? 1u : 0u);
+          for (int kk = 0; kk < 4; ++kk)   // 16 keys per step: +8 columns of P, +16 rows of V; the piece's first product overwrites O
+            mma_f16_ts(tmem + mt * kHeadDim, ap + kk * 8, dv + static_cast<uint64_t>(kk * 128), idesc_o,
+                       (i > 0 || kk > 0) ? 1u : 0u);
+        }
+        __syncwarp();
       }
-      if (!ok) {
-        fail(ctl, p.err);
-        break;
+      if (!ok) break;
+      if (elect_one()) {
+        mma_commit(&ctl->v_empty[stage]);
+        mma_commit(&ctl->s_empty[t]);   // S stage t (holding P) is free for S two units later
       }
-      mma_commit(&ctl->v_empty[stage]);
-      mma_commit(&ctl->s_empty[t]);   // S stage t (holding P) is free for S two units later
+      __syncwarp();
       if (++stage == p.kv_stages) {
         stage = 0;
-        kphase ^= 1;
+        vphase ^= 1;
       }
     }
   }
-  mma_commit(&ctl->drain);
-  mbar_wait(&ctl->drain, 0, drain_limit(p.wait_ns));
+  if (!ok) fail(ctl, p.err);
+  if (elect_one()) mma_commit(&ctl->drain);
+  warp_wait(&ctl->drain, 0, drain_limit(p.wait_ns));
 }
 
 // Maximum raw logit of a thread's row over the unit's first `lim` keys.
@@ -652,9 +660,9 @@ __global__ void __launch_bounds__(kAttnThreads, 1) k_window_attn(const __grid_co
   } else if (warp == 3) {
     if (lane == 0) v_loader(p, ctl, sV, fb, fe);
   } else if (warp == 1) {
-    if (lane == 0) mma_s_loop(p, ctl, sQ, sK, tmem, fb, fe);
+    mma_s_loop(p, ctl, sQ, sK, tmem, fb, fe);
   } else if (warp == 2) {
-    if (lane == 0) mma_pv_loop(p, ctl, sV, tmem, fb, fe);
+    mma_pv_loop(p, ctl, sV, tmem, fb, fe);
   } else if (warp >= kSoftWarp0 && warp < kSoftWarp0 + kSoftWarps) {
     const int mt = (warp - kSoftWarp0) >> 2;
     softmax_loop(p, ctl, tmem, mt, warp & 3, lane, 256 + mt * kAttnUnitKeys, 128, mt * kHeadDim, blockIdx.x, fb, fe);

@@ -76,6 +76,11 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, uint64
   }
 }
 
+// mbar_wait by a whole warp: true when every lane's succeeded.
+__device__ __forceinline__ bool warp_wait(uint64_t* bar, uint32_t parity, uint64_t limit_ns) {
+  return __all_sync(0xffffffffu, mbar_wait(bar, parity, limit_ns));
+}
+
 // ------------------------------------------------------------------ TMA
 
 // 3-D tiled load into shared memory, completion signalled on `bar` (tx bytes).
@@ -179,6 +184,22 @@ __device__ __forceinline__ void mma_bf16(uint32_t d_tmem, uint64_t adesc, uint64
       "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(d_tmem),
       "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
       : "memory");
+}
+
+// True in one lane of a fully active warp, the same one each time.  An MMA
+// issuer that runs as a whole warp and elects the lane only around the
+// instructions keeps its descriptors in uniform registers, which tcgen05.mma
+// reads; issued from a single divergent thread every product takes 60 to 77
+// cycles whatever its size (measured, K = 16: N = 64 74 -> 53 cycles, N = 128
+// 77 -> 68, A in tensor memory and N = 64 73 -> 37).
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "elect.sync _|p, 0xffffffff;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}\n"
+      : "=r"(p));
+  return p != 0;
 }
 
 // Arrives on `bar` once every tcgen05.mma issued so far by this thread is done.
