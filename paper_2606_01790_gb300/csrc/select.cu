@@ -447,6 +447,8 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_calibrate(const __grid_consta
     int nv = 0;
     uint32_t kmn = 0xFFFFFFFFu, kmx = 0u;
     float smn = 3.4e38f, smx = -3.4e38f;
+    const bool all_frames = kp.mi_span == 0;
+    bool bad = false;   // a visual token outside the patch grid
     int v = warp * span + lane - hw;
     float4 s_next = make_float4(0.f, 0.f, 0.f, 0.f);
     uint4 m_next = make_uint4(0u, 0u, 0u, 0u);
@@ -505,32 +507,34 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_calibrate(const __grid_consta
               if (t0 + i < Lp) S[t0 + i] = x[i];
           }
         }
+        // selects instead of branches: one rarely divergent branch per vector,
+        // for the current frame's tokens
         uint32_t key[4];
+        bool on[4], newest[4];
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
-          key[i] = 0u;
-          if (t0 + i >= Lp) continue;
-          smn = fminf(smn, x[i]);
-          smx = fmaxf(smx, x[i]);
-          if (!meta_visual(mw[i])) continue;
-          const int r = meta_row(mw[i]), c = meta_col(mw[i]);
-          if (r >= R || c >= C) {
-            atomicOr(st.err, kErrMeta);
-            continue;
-          }
-          const bool newest = meta_frame(mw[i]) == sv.cur_frame;
-          if (newest) atomicAdd(&cur[r * C + c], x[i]);
-          if (kp.mi_span == 0 || newest) {
-            key[i] = max(order_key(x[i]), 1u);
-            ++nv;
-            kmn = min(kmn, key[i]);
-            kmx = max(kmx, key[i]);
-          }
+          const bool in = t0 + i < Lp, vis = in && meta_visual(mw[i]);
+          const bool ok = meta_row(mw[i]) < R && meta_col(mw[i]) < C;
+          bad |= vis && !ok;
+          newest[i] = vis && ok && meta_frame(mw[i]) == sv.cur_frame;
+          on[i] = vis && ok && (all_frames || newest[i]);
+          smn = fminf(smn, in ? x[i] : smn);
+          smx = fmaxf(smx, in ? x[i] : smx);
+          key[i] = on[i] ? max(order_key(x[i]), 1u) : 0u;
+          nv += on[i];
+          kmn = min(kmn, on[i] ? key[i] : 0xFFFFFFFFu);
+          kmx = max(kmx, key[i]);
+        }
+        if (newest[0] || newest[1] || newest[2] || newest[3]) {
+#pragma unroll
+          for (int i = 0; i < 4; ++i)
+            if (newest[i]) atomicAdd(&cur[meta_row(mw[i]) * C + meta_col(mw[i])], x[i]);
         }
         if (in_smem) reinterpret_cast<uint4*>(keys)[v] = make_uint4(key[0], key[1], key[2], key[3]);
       }
       v += NW * span;
     }
+    if (bad) atomicOr(st.err, kErrMeta);
     nv = __reduce_add_sync(kFullMask, nv);
     kmn = __reduce_min_sync(kFullMask, kmn);
     kmx = __reduce_max_sync(kFullMask, kmx);
@@ -866,18 +870,17 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_calibrate(const __grid_consta
     gs += g_lo;
     z += sb;
     smx = max(smx, __float_as_uint(fmaxf(sb, 0.f)));
-    if (sb > 0.f) zl += sb * lg2_approx(sb);
+    zl += sb > 0.f ? sb * lg2_approx(sb) : 0.f;
     const float beta = (1.f - lam) + lam * static_cast<float>(G) * sh.w[gs];
-    float d = 1.f;
-    if (meta_visual(mt)) {   // Eq. (9) and its variants
-      nvs += 1.f;
-      const float df = static_cast<float>(sv.cur_frame - meta_frame(mt)), ph = sh.phi[gs];
-      float shape;
-      if (kp.decay_mode == 1) shape = fmaxf(0.f, 1.f - kp.delta * (df * ph));
-      else if (kp.decay_mode == 2) shape = powf(1.f + df * ph, -kp.delta);
-      else shape = expf(-kp.delta * df * ph);
-      d = kp.d_min + (1.f - kp.d_min) * shape;
-    }
+    // Eq. (9) and its variants, for every token; text takes D = 1
+    const bool vis = meta_visual(mt);
+    nvs += vis ? 1.f : 0.f;
+    const float df = vis ? static_cast<float>(sv.cur_frame - meta_frame(mt)) : 0.f, ph = sh.phi[gs];
+    float shape;
+    if (kp.decay_mode == 1) shape = fmaxf(0.f, 1.f - kp.delta * (df * ph));
+    else if (kp.decay_mode == 2) shape = powf(1.f + df * ph, -kp.delta);
+    else shape = expf(-kp.delta * df * ph);
+    const float d = vis ? kp.d_min + (1.f - kp.d_min) * shape : 1.f;
     const float x = fmaxf(sb * beta * d, 0.f) + 0.f;   // (no negative zero)
     xs[i] = x;
     if (B > 0) atomicAdd(&hist[sbucket(desc_key(x))], 1);
@@ -939,6 +942,44 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_calibrate(const __grid_consta
     }
     Hn = entropy(Z, ZL, SM);
     T = temperature(Hn);
+  };
+  auto write_stats = [&]() {   // by CTA 0's last warp
+    if (rank != 0 || warp != NW - 1 || !sv.stats) return;
+    float* stats = sv.stats + static_cast<int64_t>(layer) * STARKV_STATS_STRIDE(G);
+    if (lane < G) {
+      const float Hr = per_head ? entropy(sh.pz[lane], sh.pzl[lane], sh.psmax[lane]) : Hn;
+      stats[8 + lane] = sh.mi[lane];
+      stats[8 + G + lane] = sh.mib[lane];
+      stats[8 + 2 * G + lane] = sh.w[lane];
+      stats[8 + 3 * G + lane] = sh.phi[lane];
+      stats[8 + 4 * G + lane] = Hr;
+      stats[8 + 5 * G + lane] = per_head ? temperature(Hr) : T;
+    }
+    if (lane == 0) {
+      float hs = Hn, ts = T, zs = Z, nvf = sh.pv[0];
+      if (per_head) {
+        hs = ts = zs = 0.f;
+        for (int r = 0; r < G; ++r) {
+          const float Hr = entropy(sh.pz[r], sh.pzl[r], sh.psmax[r]);
+          hs += Hr;
+          ts += temperature(Hr);
+          zs += sh.pz[r];
+        }
+        hs *= 1.f / static_cast<float>(G);
+        ts *= 1.f / static_cast<float>(G);
+        zs *= 1.f / static_cast<float>(G);   // sum_t s_bar_t = mean over g of the row sums
+      } else {
+        for (int r = 1; r < ncta; ++r) nvf += sh.pv[r];
+      }
+      stats[0] = hs;
+      stats[1] = ts;
+      stats[2] = lam;
+      stats[3] = static_cast<float>(sh.n_old);
+      stats[4] = zs;
+      stats[5] = nvf;
+      stats[6] = static_cast<float>(B);
+      stats[7] = 0.f;
+    }
   };
   const int seg = ceil_div(nr, NW * 32) * 32;   // one contiguous segment per warp: warp and lane order are position order
   const int w0 = min(nr, warp * seg), w1 = min(nr, w0 + seg);
@@ -1091,6 +1132,8 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_calibrate(const __grid_consta
     const bool wait_peers = !per_head && !ties;
     if (wait_peers) cluster_arrive();
     find_T();   // while the candidates travel
+    if (!per_head) write_stats();
+    __syncwarp();
     if (wait_peers) cluster_wait();
     else __syncthreads();
     uint32_t kT = lo, tT = 0u;   // kept: key below kT, or equal to it and (at position <= tT | among the first `quota`)
@@ -1156,46 +1199,13 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_calibrate(const __grid_consta
     }
   } else {
     find_T();
+    if (!per_head) write_stats();
     const float invT = 1.f / T;
     for (int i = tid; i < nr; i += NT) score[i] = ex2_approx(invT * lg2_approx(xs[i]));
   }
-  if (per_head) cluster_wait();   // the peers' partial sums are here, and this CTA's have reached them
-  if (rank == 0 && warp == 0 && sv.stats) {
-    float* stats = sv.stats + static_cast<int64_t>(layer) * STARKV_STATS_STRIDE(G);
-    if (lane < G) {
-      const float Hr = per_head ? entropy(sh.pz[lane], sh.pzl[lane], sh.psmax[lane]) : Hn;
-      stats[8 + lane] = sh.mi[lane];
-      stats[8 + G + lane] = sh.mib[lane];
-      stats[8 + 2 * G + lane] = sh.w[lane];
-      stats[8 + 3 * G + lane] = sh.phi[lane];
-      stats[8 + 4 * G + lane] = Hr;
-      stats[8 + 5 * G + lane] = per_head ? temperature(Hr) : T;
-    }
-    if (lane == 0) {
-      float hs = Hn, ts = T, zs = Z, nvf = sh.pv[0];
-      if (per_head) {
-        hs = ts = zs = 0.f;
-        for (int r = 0; r < G; ++r) {
-          const float Hr = entropy(sh.pz[r], sh.pzl[r], sh.psmax[r]);
-          hs += Hr;
-          ts += temperature(Hr);
-          zs += sh.pz[r];
-        }
-        hs *= 1.f / static_cast<float>(G);
-        ts *= 1.f / static_cast<float>(G);
-        zs *= 1.f / static_cast<float>(G);   // sum_t s_bar_t = mean over g of the row sums
-      } else {
-        for (int r = 1; r < ncta; ++r) nvf += sh.pv[r];
-      }
-      stats[0] = hs;
-      stats[1] = ts;
-      stats[2] = lam;
-      stats[3] = static_cast<float>(sh.n_old);
-      stats[4] = zs;
-      stats[5] = nvf;
-      stats[6] = static_cast<float>(B);
-      stats[7] = 0.f;
-    }
+  if (per_head) {
+    cluster_wait();   // the peers' partial sums are here, and this CTA's have reached them
+    write_stats();
   }
 }
 
