@@ -535,6 +535,55 @@ __global__ void __launch_bounds__(kScoreThreads, 1) k_score_lse(const __grid_con
   }
 }
 
+// Pass 2's epilogue over the n tiles of a piece (the CTA's tiles jt0, jt0 + 1,
+// ...) in one warp: NCH 16-column chunks of its quarter of the columns.
+//
+// The four column quarters of a key lie in four warps.  Each writes its sum of
+// tile j to slot j mod 8 between its releases of tiles j and j + 1, so that a
+// warp that finds tile j + 3 ready (issued once all 16 warps had released tile
+// j + 1) finds all four: one warp of each lane quadrant, in turn, then adds
+// them in order and stores the row.  No warp waits for another inside a piece,
+// and one row goes to memory instead of four.  A slot is written again at tile
+// j + 8, after every warp has released tile j + 6 and so read the slot before.
+// The piece's last three tiles are stored after a barrier of the epilogue warps.
+// `dst`: this thread's key of the first tile, `left` keys of the row from it on.
+template <int NCH>
+__device__ __forceinline__ bool accum_piece(const ScoreParams& p, SmemCtl* ctl, uint32_t base0, float* sS, float* dst, int n,
+                                            int left, int jt0, int wg, int q, int quad, int lane, bool dead) {
+  const float2 sc2 = make_float2(p.scale2, p.scale2), zero2 = make_float2(0.f, 0.f);
+  float* const mine = sS + wg * kTileKeys + q;
+  auto flush = [&](int i) {   // tile i of the piece, by warpgroup (jt0 + i) mod 4
+    if (((jt0 + i) & 3) != wg) return;
+    const float* v = sS + ((jt0 + i) & (kSumSlots - 1)) * (4 * kTileKeys) + q;
+    dst[i * kTileKeys] = ((v[0] + v[kTileKeys]) + v[2 * kTileKeys]) + v[3 * kTileKeys];
+  };
+#pragma unroll 1
+  for (int i = 0; i < n; ++i) {
+    if (dead) break;
+    const int jt = jt0 + i, ts = jt & 1;
+    if (!__all_sync(kFull, mbar_wait(&ctl->t_full[ts][0], (jt >> 1) & 1, p.wait_ns))) {
+      fail(ctl, p.err);
+      dead = true;
+      break;
+    }
+    tc_fence_after();
+    float2 a0 = make_float2(0.f, 0.f), a1 = make_float2(0.f, 0.f);
+    if (NCH > 0)
+      stream16(base0 + ts * 256, NCH, [&](const uint32_t(&v)[16], int) { exp2_acc16(v, sc2, zero2, a0, a1); });
+    const float2 a = fadd2(a0, a1);
+    tc_fence_before();
+    __syncwarp();
+    if (lane == 0) mbar_arrive(&ctl->t_empty[ts]);
+    mine[(jt & (kSumSlots - 1)) * (4 * kTileKeys)] = a.x + a.y;
+    if (i >= 3) flush(i - 3);   // (a whole tile: the row goes on)
+  }
+  named_bar_sync(1, kEpiThreads);   // every warp's last sums are written (all reach this, also after a timeout)
+  if (!dead)
+    for (int i = max(0, n - 3); i < n; ++i)
+      if (i * kTileKeys < left) flush(i);
+  return dead;
+}
+
 __global__ void __launch_bounds__(kScoreThreads, 1) k_score_accum(const __grid_constant__ ScoreParams p) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = align1024(smem_raw);
@@ -576,7 +625,7 @@ __global__ void __launch_bounds__(kScoreThreads, 1) k_score_accum(const __grid_c
     const int ch0 = wg * (nc >> 2) + min(wg, nc & 3);
     const int nch = (nc >> 2) + (wg < (nc & 3) ? 1 : 0);
     const uint32_t base0 = tmem + (static_cast<uint32_t>(quad * 32) << 16) + ch0 * 16;
-    const float sc = p.scale2, isc = 1.f / p.scale2, sqd = sqrtf(static_cast<float>(kHeadDim));
+    const float isc = 1.f / p.scale2, sqd = sqrtf(static_cast<float>(kHeadDim));
     // the -lse operand of the piece `it` into buffer `buf`: window row et holds x = -lse2 / scale (= -lse sqrt(d)
     // for a supplied natural-log normaliser) as three bf16 parts (x = hi + mid
     // + lo to about 2^-24 relative) in its K columns 0..2; rows past the
@@ -605,20 +654,6 @@ __global__ void __launch_bounds__(kScoreThreads, 1) k_score_accum(const __grid_c
     };
     int jt = 0, kp = 0;
     bool dead = false;
-    // The four column quarters of a key lie in four warps.  Each writes its
-    // sum of tile j to slot j mod 8 before it releases the tile's accumulator
-    // stage, so that a warp that finds tile j + 2 ready (the stage's next
-    // product, issued once all 16 warps had released it) finds all four: one
-    // warp of each lane quadrant, in turn, then adds them in order and stores
-    // the row.  No warp waits for another, and one row goes to memory instead
-    // of four.  A slot is written again at tile j + 8, after every warp has
-    // released tile j + 6 and so read the slot long before.
-    float *pend1 = nullptr, *pend2 = nullptr;   // where this key's sums of the last two tiles go (NULL: past the row)
-    auto flush = [&](int j, float* to) {   // tile j's sums, by warpgroup j mod 4
-      if ((j & 3) != wg || to == nullptr) return;
-      const float* v = sS + (j & (kSumSlots - 1)) * (4 * kTileKeys) + q;
-      *to = ((v[0] + v[kTileKeys]) + v[2 * kTileKeys]) + v[3 * kTileKeys];
-    };
     PieceIter c(p, fb, fe);
     if (c.valid()) {
       // the ones operand: bf16 1.0 in K columns 0..2 of core matrix 0, zeros elsewhere
@@ -628,7 +663,6 @@ __global__ void __launch_bounds__(kScoreThreads, 1) k_score_accum(const __grid_c
       }
       write_x(c, 0);
     }
-    const float2 sc2 = make_float2(sc, sc), zero2 = make_float2(0.f, 0.f);
     for (; c.valid(); ++kp) {
       // the next piece's operand goes to the other buffer now, one piece
       // ahead of its MMAs (this piece's buffer was written one piece earlier;
@@ -637,35 +671,18 @@ __global__ void __launch_bounds__(kScoreThreads, 1) k_score_accum(const __grid_c
       nx.next(p);
       if (nx.valid()) write_x(nx, (kp + 1) & 1);
       const ScoreSeq& sq = p.seq[c.s];
-      int left = sq.Lp - (c.j0 * kTileKeys + q);   // > 0: this thread's key of the tile is past key
-      float* dst = sq.s_raw + static_cast<int64_t>(c.l * p.G + c.g) * raw_stride(sq.Lp) + c.j0 * kTileKeys + q;
-      for (const int jt1 = jt + c.n; jt < jt1; ++jt, left -= kTileKeys, dst += kTileKeys) {
-        if (dead) continue;
-        const int ts = jt & 1;
-        if (!__all_sync(kFull, mbar_wait(&ctl->t_full[ts][0], (jt >> 1) & 1, p.wait_ns))) {
-          fail(ctl, p.err);
-          dead = true;
-          continue;
-        }
-        tc_fence_after();
-        float2 a0 = make_float2(0.f, 0.f), a1 = make_float2(0.f, 0.f);
-        if (nch > 0)
-          stream16(base0 + ts * 256, nch, [&](const uint32_t(&v)[16], int) { exp2_acc16(v, sc2, zero2, a0, a1); });
-        const float2 a = fadd2(a0, a1);
-        sS[((jt & (kSumSlots - 1)) * 4 + wg) * kTileKeys + q] = a.x + a.y;
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&ctl->t_empty[ts]);
-        if (jt >= 2) flush(jt - 2, pend2);
-        pend2 = pend1;
-        pend1 = left > 0 ? dst : nullptr;
+      // this thread's key of the piece's first tile, in the unpooled row
+      const int key0 = c.j0 * kTileKeys + q;
+      float* dst = sq.s_raw + static_cast<int64_t>(c.l * p.G + c.g) * raw_stride(sq.Lp) + key0;
+      switch (nch) {   // this warp's 16-column chunks, the same for the whole launch
+        case 0: dead = accum_piece<0>(p, ctl, base0, sS, dst, c.n, sq.Lp - key0, jt, wg, q, quad, lane, dead); break;
+        case 1: dead = accum_piece<1>(p, ctl, base0, sS, dst, c.n, sq.Lp - key0, jt, wg, q, quad, lane, dead); break;
+        case 2: dead = accum_piece<2>(p, ctl, base0, sS, dst, c.n, sq.Lp - key0, jt, wg, q, quad, lane, dead); break;
+        case 3: dead = accum_piece<3>(p, ctl, base0, sS, dst, c.n, sq.Lp - key0, jt, wg, q, quad, lane, dead); break;
+        default: dead = accum_piece<4>(p, ctl, base0, sS, dst, c.n, sq.Lp - key0, jt, wg, q, quad, lane, dead); break;
       }
+      jt += c.n;
       c = nx;
-    }
-    named_bar_sync(1, kEpiThreads);   // every warp's last sums are written (all reach this, also after a timeout)
-    if (!dead) {
-      if (jt >= 2) flush(jt - 2, pend2);
-      if (jt >= 1) flush(jt - 1, pend1);
     }
   }
   __syncthreads();
