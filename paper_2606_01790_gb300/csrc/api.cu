@@ -384,6 +384,7 @@ starkv_status run_score(starkv_state* st, const starkv_seq* seqs, int i0, int i1
   *partial_cursor += tiles;
   p.err = st->dev.err;
   p.wait_ns = st->wait_ns;
+  p.after_lse = need_lse;
   if (need_lse)
     CUDA_TRY(launch(st, STARKV_KERNEL_SCORE_LSE, stream, [&] { return score_lse_launch(p, p.grid1, stream); }));
   CUDA_TRY(launch(st, STARKV_KERNEL_SCORE_ACCUM, stream, [&] { return score_accum_launch(p, p.grid1, stream); }));

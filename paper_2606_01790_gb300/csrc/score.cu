@@ -298,23 +298,20 @@ __device__ void mma_loop(const ScoreParams& p, SmemCtl* ctl, const uint8_t* sQ, 
   mbar_wait(&ctl->drain, 0, drain_limit(p.wait_ns));
 }
 
-// log2-domain log-sum-exp of window row `col` of the (seq, layer, group) row
-// whose first flat tile is `r0`, from the pass-1 partials of every CTA piece
-// that covered the row: one pass, eight partials loaded at a time, each batch
-// merged into the running (maximum, sum).
-__device__ float combine_lse2(const ScoreParams& p, int64_t r0, int nt, int col) {
+// (maximum, sum) in log2 units of window row `col` of the (seq, layer, group)
+// row whose first flat tile is `r0`, over the pass-1 partials of the CTA pieces
+// `c`, c + step, ... <= c1 that covered it: eight partials loaded at a time,
+// each batch merged into the running pair.
+__device__ float2 combine_partials(const ScoreParams& p, int64_t r0, int c, int c1, int step, int col) {
   const int64_t T = p.total_tiles;
   const int P = p.grid1;
-  const int64_t r1 = r0 + nt - 1;
-  const int c0 = static_cast<int>(((r0 + 1) * P - 1) / T);
-  const int c1 = static_cast<int>(((r1 + 1) * P - 1) / T);
   float mx = -INFINITY, sum = 0.f;
-  for (int cb = c0; cb <= c1; cb += 8) {
+  for (; c <= c1; c += 8 * step) {
     float2 v[8];
 #pragma unroll
     for (int k = 0; k < 8; ++k) {
       v[k] = make_float2(-INFINITY, 0.f);
-      if (cb + k <= c1) v[k] = p.partials[max(range_begin(T, cb + k, P), r0) * kMaxRows + col];
+      if (c + k * step <= c1) v[k] = p.partials[max(range_begin(T, c + k * step, P), r0) * kMaxRows + col];
     }
     float bm = mx;
 #pragma unroll
@@ -327,7 +324,7 @@ __device__ float combine_lse2(const ScoreParams& p, int64_t r0, int nt, int col)
     mx = bm;
     sum = bs;
   }
-  return mx + log2f(sum);
+  return make_float2(mx, sum);
 }
 
 // Streams `n` 16-column chunks of this thread's TMEM lane from `base`, one
@@ -460,9 +457,11 @@ __global__ void __launch_bounds__(kScoreThreads, 1) k_score_lse(const __grid_con
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  // the set-up above overlaps the previous kernel's tail; its outputs are read below
-  griddep_launch_dependents();
+  // the set-up above overlaps the previous kernel's tail; its outputs are read
+  // below.  Pass 2 may start once every CTA is past this wait: whatever wrote K
+  // and Q is then complete, and pass 2 loads them without waiting for pass 1.
   griddep_wait();
+  griddep_launch_dependents();
   const uint32_t tmem = ctl->tmem_base;
   const int64_t T = p.total_tiles;
   const int64_t fb = range_begin(T, blockIdx.x, gridDim.x);
@@ -604,9 +603,11 @@ __global__ void __launch_bounds__(kScoreThreads, 1) k_score_accum(const __grid_c
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  // the set-up above overlaps the previous kernel's tail; its outputs are read below
+  // the set-up above overlaps the previous kernel's tail; its outputs are read
+  // by the epilogue warps.  K and Q are loaded right away when that kernel is
+  // this call's pass 1 (p.after_lse), which waited for whatever wrote them.
   griddep_launch_dependents();
-  griddep_wait();
+  if (!p.after_lse || warp >= kEpiWarp0) griddep_wait();
   const uint32_t tmem = ctl->tmem_base;
   const int64_t T = p.total_tiles;
   const int64_t fb = range_begin(T, blockIdx.x, gridDim.x);
@@ -626,18 +627,42 @@ __global__ void __launch_bounds__(kScoreThreads, 1) k_score_accum(const __grid_c
     const int nch = (nc >> 2) + (wg < (nc & 3) ? 1 : 0);
     const uint32_t base0 = tmem + (static_cast<uint32_t>(quad * 32) << 16) + ch0 * 16;
     const float isc = 1.f / p.scale2, sqd = sqrtf(static_cast<float>(kHeadDim));
+    int jt = 0, kp = 0;
+    bool dead = false;
     // the -lse operand of the piece `it` into buffer `buf`: window row et holds x = -lse2 / scale (= -lse sqrt(d)
     // for a supplied natural-log normaliser) as three bf16 parts (x = hi + mid
     // + lo to about 2^-24 relative) in its K columns 0..2; rows past the
     // group's window rows get a large negative x (exp2 -> 0)
     auto write_x = [&](const PieceIter& it, int buf) {
+      const float* lse = p.seq[it.s].lse;
+      float2 part = make_float2(-INFINITY, 0.f);
+      if (!lse) {
+        const int64_t r0 = it.f - it.j0;   // the row's first flat tile
+        const int c0 = static_cast<int>(((r0 + 1) * p.grid1 - 1) / T);
+        const int c1 = static_cast<int>(((r0 + it.nt) * p.grid1 - 1) / T);
+        // a row spread over many CTAs (few rows in the launch): two threads per
+        // window row take every other piece, merged through a slot of sums
+        // that no tile near this one uses
+        const bool split = c1 - c0 >= 8;   // the same in every thread
+        const int col = et & (kMaxRows - 1), odd = et >> 8;
+        if (col < p.rows && (split || !odd)) part = combine_partials(p, r0, c0 + odd, c1, split ? 2 : 1, col);
+        if (split) {
+          float2* buf2 = reinterpret_cast<float2*>(sS + ((jt + 1) & (kSumSlots - 1)) * (4 * kTileKeys));
+          if (odd) buf2[col] = part;
+          named_bar_sync(1, kEpiThreads);
+          if (!odd && col < p.rows) {
+            const float2 o = buf2[col];
+            const float mx = fmaxf(part.x, o.x);   // (piece c0 has keys: finite)
+            part.y = part.y * exp2f(part.x - mx) + (o.x == -INFINITY ? 0.f : o.y * exp2f(o.x - mx));
+            part.x = mx;
+          }
+        }
+      }
       if (et < p.n2) {
         float x = -3.0e38f;
-        if (et < p.rows) {
-          const float* lse = p.seq[it.s].lse;
+        if (et < p.rows)
           x = lse ? -lse[(static_cast<int64_t>(p.layer0 + it.l) * p.G + it.g) * p.rows + et] * sqd
-                  : -combine_lse2(p, it.f - it.j0, it.nt, et) * isc;
-        }
+                  : -(part.x + log2f(part.y)) * isc;
         const __nv_bfloat16 hi = __float2bfloat16_rn(x);
         const float r1 = x - __bfloat162float(hi);
         const __nv_bfloat16 mid = __float2bfloat16_rn(r1);
@@ -652,8 +677,6 @@ __global__ void __launch_bounds__(kScoreThreads, 1) k_score_accum(const __grid_c
       named_bar_sync(1, kEpiThreads);
       if (et == 0) mbar_arrive(&ctl->x_full[buf]);
     };
-    int jt = 0, kp = 0;
-    bool dead = false;
     PieceIter c(p, fb, fe);
     if (c.valid()) {
       // the ones operand: bf16 1.0 in K columns 0..2 of core matrix 0, zeros elsewhere

@@ -27,6 +27,7 @@ struct ScoreParams {
   int n_mtiles;        // ceil(rows / 128) (pass-1 M tiles)
   int q_rows;          // shared-memory Q rows per 64-column half (= n2)
   int kstages;         // K-tile pipeline depth (from the shared-memory budget)
+  int after_lse;       // pass 2 follows this call's pass 1
   int grid1;           // pass-1 grid size (defines the partial-slot partition)
   int64_t total_tiles;
   float scale2;        // log2(e) / sqrt(d)
