@@ -19,9 +19,9 @@
 //   MI EMA, min-max and softmax prior, lambda schedule                  (Eqs. 6-7);
 //   s_bar, g*, Z = sum s_bar, the entropy H (Sec. 3.6) and x_t =
 //     max(s_bar beta D, 0), with its bucket counted in the same pass: the
-//     4096 buckets span the range that the groups' extremes and the factors'
-//     bounds allow (values outside fall into the end buckets), so no exchange
-//     of the actual range is needed first;
+//     4096 buckets span 14 octaves below a bound from the groups' largest S
+//     (values outside fall into the end buckets), so no exchange of the actual
+//     range is needed first;
 //   global top-B with ties to the lower index (Sec. 3.7): every CTA sends its
 //     128 coarse counts (32 buckets each) and its partial sums to its peers;
 //     the coarse bucket that holds the B-th token is found on their sum, its
@@ -140,9 +140,8 @@ __device__ void warp_find_256(const int* hist, int rank, int* digit, int* below)
 
 struct CalShared {
   // ---- phase 1 (this CTA's current group)
-  int nvis;                        // tokens of the MI span
-  uint32_t kmin, kmax;             // their key range
-  uint32_t smin, smax;             // key range of the whole row
+  uint32_t kmin, kmax;             // key range of the MI span: the smallest key - 1 and the largest
+  uint32_t smax;                   // the whole row's largest
   uint32_t slots;                  // boundary buckets so far: count in bits 24.., their tokens below
   int slot_off[kMaxTargets + 1];   // slot -> first entry of its candidates in the pool
   int slot_n[kMaxTargets + 1];     // slot -> tokens in its bucket
@@ -158,7 +157,7 @@ struct CalShared {
   int eqw[32][kMaxTargets];        // keys equal to each boundary before each warp's segment
   // ---- written by every CTA of the cluster
   float mi[kMaxGroups], phi[kMaxGroups];
-  uint32_t gmin[kMaxGroups], gmax[kMaxGroups];
+  uint32_t gmax[kMaxGroups];
   float pz[kMaxCluster], pzl[kMaxCluster], pv[kMaxCluster];
   uint32_t psmax[kMaxCluster];
   uint32_t rlo[kMaxCluster], rhi[kMaxCluster];
@@ -347,10 +346,8 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_calibrate(const __grid_consta
   // block-wide counters, histograms and the current-frame row of the next group
   auto reset = [&]() {
     if (tid == 0) {
-      sh.nvis = 0;
       sh.kmin = 0xFFFFFFFFu;
       sh.kmax = 0u;
-      sh.smin = 0xFFFFFFFFu;
       sh.smax = 0u;
       sh.slots = 0u;
     }
@@ -444,33 +441,41 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_calibrate(const __grid_consta
     const bool src16 = (reinterpret_cast<uintptr_t>(src) & 15) == 0, s16 = (reinterpret_cast<uintptr_t>(S) & 15) == 0;
     const bool m16 = (reinterpret_cast<uintptr_t>(meta) & 15) == 0;
     const int nvec = (Lp + 3) >> 2;
-    int nv = 0;
-    uint32_t kmn = 0xFFFFFFFFu, kmx = 0u;
-    float smn = 3.4e38f, smx = -3.4e38f;
+    // fields of a metadata word compared in place
+    const uint32_t row_end = static_cast<uint32_t>(R) << 10, frame_now = static_cast<uint32_t>(sv.cur_frame) << 20;
     const bool all_frames = kp.mi_span == 0;
+    uint32_t kmn = 0xFFFFFFFFu, kmx = 0u;
+    float smx = -3.4e38f;
     bool bad = false;   // a visual token outside the patch grid
     int v = warp * span + lane - hw;
     float4 s_next = make_float4(0.f, 0.f, 0.f, 0.f);
     uint4 m_next = make_uint4(0u, 0u, 0u, 0u);
     auto load = [&](int v) {
       const int t0 = 4 * max(0, min(nvec - 1, v));
+      const bool whole = t0 + 3 < Lp;
       const int t1 = min(t0 + 1, Lp - 1), t2 = min(t0 + 2, Lp - 1), t3 = min(t0 + 3, Lp - 1);
-      if (m16 && t0 + 3 < Lp) m_next = *reinterpret_cast<const uint4*>(meta + t0);
+      if (m16 && whole) m_next = *reinterpret_cast<const uint4*>(meta + t0);
       else m_next = make_uint4(meta[t0], meta[t1], meta[t2], meta[t3]);
-      if (src16 && t0 + 3 < Lp) s_next = *reinterpret_cast<const float4*>(src + t0);
+      if (src16 && whole) s_next = *reinterpret_cast<const float4*>(src + t0);
       else s_next = make_float4(src[t0], src[t1], src[t2], src[t3]);
     };
     if (Lp > 0) load(v);
 #pragma unroll 1
     for (int base = warp * span; base < nvec; base += NW * span) {
       float x[4] = {s_next.x, s_next.y, s_next.z, s_next.w};
-      const uint32_t mw[4] = {m_next.x, m_next.y, m_next.z, m_next.w};
+      uint32_t mw[4] = {m_next.x, m_next.y, m_next.z, m_next.w};
       const int t0 = 4 * v;
       load(v + NW * span);
-      if (pool_here) {
+      // past the row's ends: zeros, and no visual token
+      if (static_cast<uint32_t>(t0) + 3u >= static_cast<uint32_t>(Lp)) {
 #pragma unroll
         for (int i = 0; i < 4; ++i)
-          if (t0 + i < 0 || t0 + i >= Lp) x[i] = 0.f;
+          if (static_cast<uint32_t>(t0 + i) >= static_cast<uint32_t>(Lp)) {
+            x[i] = 0.f;
+            mw[i] = 0u;
+          }
+      }
+      if (pool_here) {
         float o[4];
         if (half == 2) {   // the default window
           const float l2 = __shfl_up_sync(kFullMask, x[2], 1), l1 = __shfl_up_sync(kFullMask, x[3], 1);
@@ -510,19 +515,19 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_calibrate(const __grid_consta
         // selects instead of branches: one rarely divergent branch per vector,
         // for the current frame's tokens
         uint32_t key[4];
-        bool on[4], newest[4];
+        bool newest[4];
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
-          const bool in = t0 + i < Lp, vis = in && meta_visual(mw[i]);
-          const bool ok = meta_row(mw[i]) < R && meta_col(mw[i]) < C;
-          bad |= vis && !ok;
-          newest[i] = vis && ok && meta_frame(mw[i]) == sv.cur_frame;
-          on[i] = vis && ok && (all_frames || newest[i]);
-          smn = fminf(smn, in ? x[i] : smn);
-          smx = fmaxf(smx, in ? x[i] : smx);
-          key[i] = on[i] ? max(order_key(x[i]), 1u) : 0u;
-          nv += on[i];
-          kmn = min(kmn, on[i] ? key[i] : 0xFFFFFFFFu);
+          const bool vis = meta_visual(mw[i]);
+          const bool in = vis && (mw[i] & 0xFFC00u) < row_end && (mw[i] & 0x3FFu) < static_cast<uint32_t>(C);
+          bad |= vis && !in;
+          newest[i] = in && (mw[i] & 0x7FF00000u) == frame_now;
+          const bool on = all_frames ? in : newest[i];
+          smx = fmaxf(smx, x[i]);
+          // (the unpooled sums are sums of exponentials, so not negative)
+          const uint32_t ok = pool_here ? __float_as_uint(x[i]) | 0x80000000u : max(order_key(x[i]), 1u);
+          key[i] = on ? ok : 0u;
+          kmn = min(kmn, key[i] - 1u);
           kmx = max(kmx, key[i]);
         }
         if (newest[0] || newest[1] || newest[2] || newest[3]) {
@@ -535,23 +540,20 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_calibrate(const __grid_consta
       v += NW * span;
     }
     if (bad) atomicOr(st.err, kErrMeta);
-    nv = __reduce_add_sync(kFullMask, nv);
-    kmn = __reduce_min_sync(kFullMask, kmn);
+    kmn = __reduce_min_sync(kFullMask, kmn);   // (the smallest key - 1)
     kmx = __reduce_max_sync(kFullMask, kmx);
-    const uint32_t rmn = __reduce_min_sync(kFullMask, order_key(smn)), rmx = __reduce_max_sync(kFullMask, order_key(smx));
+    const uint32_t rmx = __reduce_max_sync(kFullMask, order_key(smx));
     if (lane == 0) {
-      atomicAdd(&sh.nvis, nv);
       atomicMin(&sh.kmin, kmn);
       atomicMax(&sh.kmax, kmx);
-      atomicMin(&sh.smin, rmn);
       atomicMax(&sh.smax, rmx);
     }
     __syncthreads();
-    const int N = sh.nvis;
+    const bool some = sh.kmax != 0u;   // the MI span holds a token
     // Sec. 3.4 RankBin: 4096 buckets spread linearly over the span's key range
     // (monotone in the key, so bucket order is key order)
     const Row row = {in_smem ? keys : nullptr, S, meta, Lp, R, C, M, sv.cur_frame, kp.mi_span, kp.inv_R, kp.inv_C,
-                     sh.kmin, 4096.f / (static_cast<float>(sh.kmax - sh.kmin) + 1.f)};
+                     sh.kmin + 1u, 4096.f / (static_cast<float>(sh.kmax - (sh.kmin + 1u)) + 1.f)};
     // every token of the MI span: f(token, key, metadata word).  A row that is
     // not on chip is read again from S, four tokens' loads at a time.
     auto each_span = [&](auto with_meta, auto&& f) {
@@ -584,7 +586,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_calibrate(const __grid_consta
         }
       }
     };
-    if (N > 0) each_span(std::false_type(), [&](int, uint32_t u, uint32_t) { atomicAdd(&hist[row.bucket(u)], 1); });
+    if (some) each_span(std::false_type(), [&](int, uint32_t u, uint32_t) { atomicAdd(&hist[row.bucket(u)], 1); });
     // ---- Sec. 3.5: the sums of phi_g = cos(current row, m_g)
     mrow = st.m + static_cast<int64_t>(sl * G + g) * RC;
     float dot = 0.f, ncur = 0.f, nm = 0.f;
@@ -602,23 +604,16 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_calibrate(const __grid_consta
     }
     __syncthreads();
     float acc = 0.f;   // this thread's part of N MI_g
-    if (N > 0) {
+    int N = 0;
+    if (some) {
       // ---- bucket table: the first rank of every bucket by a scan, then the
       // bin floor(rank K / N) of its first and last token.  One bin: every
       // token goes there.  Otherwise the bucket gets a slot and its tokens are
       // ranked among themselves.
       constexpr int kPer = kBuckets / NT;
-      const float fN = static_cast<float>(N), kn = static_cast<float>(K) / fN;
-      auto bin_of = [&](int r) {   // floor(r K / N): an estimate good to one, corrected in integers (r K < 2^28)
-        int q = static_cast<int>(static_cast<float>(r) * kn);
-        const int rk = r * K;
-        q += (q + 1) * N <= rk;
-        q -= q * N > rk;
-        return q;
-      };
+      int h[kPer];
+      int sum = 0;
       {
-        int h[kPer];
-        int sum = 0;
 #pragma unroll
         for (int k = 0; k < kPer; k += 4) {
           const int4 q = reinterpret_cast<const int4*>(hist)[(tid * kPer + k) >> 2];
@@ -628,12 +623,22 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_calibrate(const __grid_consta
           h[k + 3] = q.w;
           sum += (q.x + q.y) + (q.z + q.w);
         }
-        const int incl = warp_incl_scan(sum, lane);
-        if (lane == 31) sh.wsum[warp] = incl;
-        __syncthreads();
-        const int wv = lane < NW ? sh.wsum[lane] : 0;
-        const int wbase = __shfl_sync(kFullMask, warp_incl_scan(wv, lane) - wv, warp);
-        int first = wbase + incl - sum;
+      }
+      const int incl = warp_incl_scan(sum, lane);
+      if (lane == 31) sh.wsum[warp] = incl;
+      __syncthreads();
+      const int wincl = warp_incl_scan(lane < NW ? sh.wsum[lane] : 0, lane);
+      N = __shfl_sync(kFullMask, wincl, 31);
+      int first = (warp ? __shfl_sync(kFullMask, wincl, warp - 1) : 0) + incl - sum;
+      const float fN = static_cast<float>(N), kn = static_cast<float>(K) / fN;
+      auto bin_of = [&](int r) {   // floor(r K / N): an estimate good to one, corrected in integers (r K < 2^28)
+        int q = static_cast<int>(static_cast<float>(r) * kn);
+        const int rk = r * K;
+        q += (q + 1) * N <= rk;
+        q -= q * N > rk;
+        return q;
+      };
+      {
         uint32_t packed[kPer / 4];
         const int b0 = sum > 0 ? bin_of(first) : 0;
         if (sum == 0 || bin_of(first + sum - 1) == b0) {
@@ -724,7 +729,6 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_calibrate(const __grid_consta
     if (warp == 0 && lane < ncta) {
       dsmem_st_u32(dsmem_map(&sh.mi[g], lane), __float_as_uint(mi));
       dsmem_st_u32(dsmem_map(&sh.phi[g], lane), __float_as_uint(phi));
-      dsmem_st_u32(dsmem_map(&sh.gmin[g], lane), sh.smin);
       dsmem_st_u32(dsmem_map(&sh.gmax[g], lane), sh.smax);
     }
     if (g + ncta < G) {   // the next group of this CTA starts from clean arrays
@@ -779,7 +783,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_calibrate(const __grid_consta
   // schedule.  The same arithmetic in every CTA; CTA 0 stores the new state.
   // warp 0, lane gg < G: group gg's MI and its EMA, then the min-max and the
   // softmax over the groups by warp reductions; last, the bucket range of the
-  // selection: a bound on x_t from the extremes of S and of the factors
+  // selection: below a bound on x_t from the largest S and the largest factor
   static_assert(kMaxGroups <= 32, "one lane per group");
   if (warp == 0) {
     const int n = sh.n_old;
@@ -802,14 +806,13 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_calibrate(const __grid_consta
     const float exs = warp_sum(ex);
     if (on) sh.w[lane] = ex / exs;
     const bool mine = per_head ? lane == rank : on;
-    const float slo = order_value(__reduce_min_sync(kFullMask, mine ? sh.gmin[lane] : 0xFFFFFFFFu));
     const float shi = order_value(__reduce_max_sync(kFullMask, mine ? sh.gmax[lane] : 0u));
     if (lane == 0) {
       const float lam = sh.lam;
-      // (values outside the bound fall into the end buckets)
-      float xlo = slo * fmaxf(1.f - lam, 0.1f) * fmaxf(kp.d_min, 0.05f);
-      float xhi = shi * ((1.f - lam) + lam * static_cast<float>(G));
-      if (!(xlo >= 0.f && xlo < xhi && xhi < 3.0e38f)) {   // unusual scores: the whole range
+      // 14 octaves below a bound on the largest score (values outside fall
+      // into the end buckets)
+      float xhi = shi * ((1.f - lam) + lam * static_cast<float>(G)), xlo = xhi * 6.1e-5f;
+      if (!(xlo > 0.f && xhi < 3.0e38f)) {   // unusual scores: the whole range
         xlo = 0.f;
         xhi = 3.0e38f;
       }
