@@ -9,6 +9,7 @@ built, importing the first call raises.
 from __future__ import annotations
 
 import ctypes as C
+import struct
 from dataclasses import dataclass, fields
 from pathlib import Path
 from typing import List, Optional, Sequence
@@ -201,14 +202,6 @@ def meta_tensor(words: np.ndarray) -> torch.Tensor:
     return torch.from_numpy(np.ascontiguousarray(words).view(np.int32))
 
 
-def _ptr(t: Optional[torch.Tensor]) -> Optional[int]:
-    if t is None:
-        return None
-    if not t.is_contiguous():
-        raise ValueError("tensors must be contiguous")
-    return t.data_ptr()
-
-
 @dataclass
 class Seq:
     """One sequence of a call (``starkv_seq``).  Tensor layouts as in starkv.h."""
@@ -245,15 +238,45 @@ class Seq:
         return s
 
 
+# The fields of ``starkv_seq`` in order, packed in one go: a call marshals its
+# sequences every time (nothing is kept of them), and one ctypes attribute store
+# per field cost more than the launch it led to.  Values that do not pack go
+# through ``Seq.to_c``, with ctypes' own conversions and errors.
+_SEQ = struct.Struct("@4Pq4i7Pq3P")
+assert _SEQ.size == C.sizeof(CSeq)
+
+
+def _ptr(t: Optional[torch.Tensor]) -> int:
+    if t is None:
+        return 0
+    if not t.is_contiguous():
+        raise ValueError("tensors must be contiguous")
+    return t.data_ptr()
+
+
+def _pack_seq(s: Seq) -> bytes:
+    ptr = _ptr
+    try:
+        return _SEQ.pack(ptr(s.k), ptr(s.v), ptr(s.q), ptr(s.meta), s.meta_layer_stride, s.L, s.cur_frame, s.budget,
+                         s.slot, ptr(s.k_out), ptr(s.v_out), ptr(s.meta_out), ptr(s.idx), ptr(s.S), ptr(s.score),
+                         ptr(s.stats), s.meta_group_stride, ptr(s.lse), ptr(s.attn_o), ptr(s.attn_lse))
+    except struct.error:
+        return bytes(s.to_c())
+
+
 def _seq_array(seqs: Sequence[Seq]):
-    arr = (CSeq * max(1, len(seqs)))()
-    for i, s in enumerate(seqs):
-        arr[i] = s.to_c()
-    return arr
+    """The ``starkv_seq`` array of a call (one entry for an empty batch)."""
+    buf = b"".join([_pack_seq(s) for s in seqs]) or bytes(_SEQ.size)
+    return (CSeq * (len(buf) // _SEQ.size)).from_buffer_copy(buf)
+
+
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
 
 
 def _stream(stream) -> int:
     if stream is None:
+        if torch.cuda.is_initialized() and _raw_stream is not None:
+            return _raw_stream(torch.cuda.current_device())
         return torch.cuda.current_stream().cuda_stream if torch.cuda.is_available() else 0
     return stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
 

@@ -123,3 +123,20 @@ def test_slot_calls_check_their_arguments_on_the_host(library):
     buf = (ctypes.c_uint8 * 64)()
     assert library.starkv_export_slot(None, 0, buf, 64, None) == sk.ERR_INVALID_ARG
     assert library.starkv_import_slot(None, 0, buf, 64, None) == sk.ERR_INVALID_ARG
+
+
+def test_packed_sequences_equal_the_ctypes_struct():
+    """The one-call packing of ``starkv_seq`` gives the bytes that setting the
+    ctypes fields gives, falls back to ctypes' conversions for values that do
+    not pack, and an empty batch has one zero entry."""
+    import torch
+    t = [torch.zeros(4) for _ in range(14)]
+    full = sk.Seq(k=t[0], v=t[1], q=t[2], meta=t[3], meta_layer_stride=-(1 << 40), L=7, cur_frame=2047, budget=5, slot=3,
+                  k_out=t[4], v_out=t[5], meta_out=t[6], idx=t[7], S=t[8], score=t[9], stats=t[10],
+                  meta_group_stride=1 << 33, lse=t[11], attn_o=t[12], attn_lse=t[13])
+    for seq in (full, sk.Seq(), sk.Seq(L=1 << 31)):
+        assert bytes(sk._seq_array([seq])) == bytes(seq.to_c())
+    assert bytes(sk._seq_array([full, sk.Seq()])) == bytes(full.to_c()) + bytes(sk.CSeq())
+    assert bytes(sk._seq_array([])) == bytes(sk.CSeq())
+    with pytest.raises(ValueError):
+        sk._seq_array([sk.Seq(k=torch.zeros(4, 4).t())])
