@@ -16,14 +16,12 @@
 // both in flat order) and k_attn_combine merges the pieces of each row.
 //
 // Per unit on tcgen05, with two 128-row M tiles for up to 256 window rows:
-//   S = Q K^T           M = 128 rows, N = 64 keys, K = d, bf16 -> fp32 in TMEM
-//                       (two S stages, so the MMA of unit u+1 runs under the
-//                       softmax of unit u);
-//   softmax             rows on TMEM lanes, one thread per row: S read in two
-//                       halves (the second half's loads under the first half's
-//                       arithmetic), p = exp2(S c - m), l += p in fp32, P
-//                       rounded to fp16 and written over the first 32 of the
-//                       unit's 64 S columns (two fp16 per 32-bit column);
+//   S = Q K^T           M = 128 rows, N = 64 keys, K = d, bf16 -> fp32 in TMEM;
+//   softmax             rows on TMEM lanes, one thread per row: S into registers
+//                       (which frees its stage: S of the next unit runs under
+//                       the arithmetic), the row maximum, p = exp2(S c - m),
+//                       l += p in fp32, P rounded to fp16 and stored beside S
+//                       (two fp16 per 32-bit column);
 //   O += P V            M = 128, N = d = 128, K = 64 keys, fp16 -> fp32 in TMEM,
 //                       A = P read from tensor memory;
 //                       V arrives as bf16 and four warps convert it to fp16 in
@@ -32,15 +30,24 @@
 // The row reference m is the piece's first unit's maximum and moves only when
 // a unit's maximum exceeds it by more than 15 (fp16 holds P < 2^16); the move
 // rescales that row's O in TMEM after the previous unit's P V is done (rare).
-// Later units take no maximum unless their sum of P exceeds 2^15: below that
-// no p can exceed 2^15, so no reference can have to move.
-// An S stage holds P until the P V product of its unit is done, which frees
-// it for S two units later.  Warp roles: warp 0 loads K (a four-stage ring,
-// each stage free once S of its unit is done) and Q per piece, warp 3 loads V
-// (a four-stage ring, free once the P V product is done), warp 1 issues S and
-// owns TMEM, warp 2 issues P V, warps 4..11 softmax (warpgroup = M tile),
-// warps 12..15 V conversion.
+//
+// With two M tiles the kernel is bound by the shared memory's bandwidth: with
+// both operands of S there, a unit moved 192 KB (S 96, P V 32, the conversion 32,
+// the loads 32), 2030 cycles at the 91 to 95 bytes a clock it reaches, where HBM
+// needs 1420.  So the queries are the A operand in tensor memory as far as that
+// has room: O 256 columns, S 128, P 64, which leaves half of their 64 a tile
+// (160 KB a unit).  Measured (28 query and 4 KV heads, window 32, 28 layers x
+// 14,000 tokens): 168 -> 157 us.  All the queries there and S and P sharing one
+// stage: 181 (S of the next unit waits for P V); all of them and one S stage for
+// both M tiles: 172.  One M tile has room for all the queries and is near the
+// HBM rate either way (32 and 8 heads, window 16: 67 us).
+// Five- and six-stage rings were slower than four (by 1 and 3 us).
+// Warp roles: warp 0 loads K (a four-stage ring, each stage free once S of its
+// unit is done) and Q per piece, warp 3 loads V (a four-stage ring, free once
+// the P V product is done), warp 1 issues S and owns TMEM, warp 2 issues P V,
+// warps 4..11 softmax (warpgroup = M tile), warps 12..15 V conversion.
 #include <algorithm>
+#include <type_traits>
 #include <utility>
 
 #include <cuda_fp16.h>
@@ -56,7 +63,7 @@ namespace {
 constexpr int kStages = 4;                        // largest depth of the K ring and of the V ring
 constexpr int kUnitBytes = kAttnUnitKeys * 256;   // 64 keys x 128 bf16: 16 KB (K or V)
 constexpr int kHalfBytes = kAttnUnitKeys * 128;   // one 64-column half of a unit: 8 KB
-constexpr int kTmemCols = 512;                    // O [0, 256), S stage t at 256 + 128 t
+constexpr int kTmemCols = 512;
 constexpr int kSoftWarp0 = 4, kSoftWarps = 8;
 constexpr int kConvWarp0 = 12, kConvWarps = 4;
 constexpr uint32_t kFull = 0xffffffffu;
@@ -71,10 +78,11 @@ __device__ __forceinline__ uint64_t drain_limit(uint64_t wait_ns) {
 struct AttnCtl {
   uint64_t k_full[kStages], k_empty[kStages];
   uint64_t v_full[kStages], v_empty[kStages], v_ready[kStages];
-  uint64_t s_full[2][2];   // [stage][M tile]: S of that M tile is in the stage
-  uint64_t s_empty[2];      // the stage's P V products are done
-  uint64_t p_full[2][2];    // [stage][M tile]: P of that M tile is written
-  uint64_t q_full, q_empty, drain;
+  uint64_t s_full[2], s_empty[2];   // [unit's line]: S is in its stage; its softmax warps have read it
+  uint64_t p_full[2], p_empty[2];   // P is written; the P V product is done
+  uint64_t q_full, q_empty; // a piece's queries are in shared memory; every softmax warp has read its rows
+  uint64_t qt_full;         // ... and has them in tensor memory
+  uint64_t drain;
   uint32_t tmem_base;
   volatile int abort;
 };
@@ -264,48 +272,64 @@ __device__ void v_loader(const AttnParams& p, AttnCtl* ctl, uint8_t* sV, int64_t
       if (last_ph[i] >= 0) mbar_wait(&ctl->v_full[i], last_ph[i], drain_limit(p.wait_ns));
 }
 
-// Two MMA issuers walk the same units: warp 1 issues S(u) into S stage u & 1
-// as soon as the stage is free and K(u) has landed, warp 2 issues
-// O += P(u) V(u) once the softmax has written P(u) and V(u) is fp16, so that
-// S of the next units runs ahead of the products.  Each runs as a whole warp
-// (elect_one).
-__device__ void mma_s_loop(const AttnParams& p, AttnCtl* ctl, const uint8_t* sQ, const uint8_t* sK, uint32_t tmem,
-                           int64_t fb, int64_t fe) {
+// A line is what a softmax warpgroup works through in order: with two M tiles
+// their units, one line each; with one M tile its even and odd units.  A line
+// has its own barriers, S stage and P.  Tensor memory, in columns: O of M tile m
+// at 128 m, the S stages (64 each) and P (32 each) of the lines, and from 448 on
+// the queries of K steps 0 .. kTsSteps - 1 (8 columns a step and M tile).
+template <bool TWO>
+struct Tmem {
+  static constexpr int kTsSteps = TWO ? 4 : 8;   // K steps (of 8) whose queries are in tensor memory
+  static __device__ __forceinline__ uint32_t o(int mt) { return mt * kHeadDim; }
+  static __device__ __forceinline__ uint32_t s(int line) { return 256 + 64 * line; }
+  static __device__ __forceinline__ uint32_t p(int line) { return 384 + 32 * line; }
+  static __device__ __forceinline__ uint32_t q(int mt) { return 448 + 32 * mt; }
+  // unit ui of M tile mt: its line, and the parity of its use of the line
+  static __device__ __forceinline__ int line(uint32_t ui, int mt) { return TWO ? mt : static_cast<int>(ui & 1); }
+  static __device__ __forceinline__ uint32_t par(uint32_t ui) { return TWO ? ui & 1 : (ui >> 1) & 1; }
+};
+
+// Two MMA issuers walk the same units: warp 1 issues S(u) as soon as the S stage
+// is free and K(u) has landed, warp 2 issues O += P(u) V(u) once the softmax has
+// written P(u) and V(u) is fp16.  Each runs as a whole warp (elect_one): issued
+// from one divergent thread a product took 60 to 77 cycles whatever its size.
+template <bool TWO>
+__device__ void mma_s_loop(const AttnParams& p, AttnCtl* ctl, const uint8_t* sQ, const uint8_t* sK, uint32_t tmem, int64_t fb,
+                           int64_t fe) {
+  using T = Tmem<TWO>;
   const uint32_t idesc_s = idesc_bf16(128, kAttnUnitKeys);
-  const uint64_t dq0 = sdesc_k_sw128(smem_u32(sQ)), dk0 = sdesc_k_sw128(smem_u32(sK));
-  const uint32_t qhalf16 = (p.q_rows * 128) >> 4;
+  const uint64_t dk0 = sdesc_k_sw128(smem_u32(sK));
+  const uint64_t dq1 = sdesc_k_sw128(smem_u32(sQ) + p.q_rows * 128);   // the queries' second half
   int stage = 0, kphase = 0, pc = 0;
   uint32_t ui = 0;
   bool ok = true;
   for (PieceIter c(p, fb, fe); ok && c.valid(); c.next(p)) {
-    ok = !__any_sync(kFull, ctl->abort) && warp_wait(&ctl->q_full, pc & 1, p.wait_ns);
+    ok = !__any_sync(kFull, ctl->abort) && warp_wait(&ctl->qt_full, pc & 1, p.wait_ns);
     ++pc;
     for (int i = 0; ok && i < c.n; ++i, ++ui) {
-      const int t = static_cast<int>(ui & 1);
-      ok = warp_wait(&ctl->k_full[stage], kphase, p.wait_ns) &&
-           warp_wait(&ctl->s_empty[t], ((ui >> 1) & 1) ^ 1, p.wait_ns);
-      if (!ok) break;
-      tc_fence_after();
+      ok = warp_wait(&ctl->k_full[stage], kphase, p.wait_ns);
       const uint64_t dk = dk0 + static_cast<uint64_t>(stage * (kUnitBytes >> 4));
-      if (elect_one()) {
 #pragma unroll
-        for (int mt = 0; mt < 2; ++mt) {
-          if (mt >= p.n_mtiles) break;
-          // M tile 1 reads rows 128..255 of each Q half; rows past q_rows feed
-          // accumulator rows that no thread reads
-          const uint64_t dq = dq0 + static_cast<uint64_t>(mt * ((128 * 128) >> 4));
+      for (int mt = 0; mt < (TWO ? 2 : 1); ++mt) {
+        const int ln = T::line(ui, mt);
+        ok = ok && warp_wait(&ctl->s_empty[ln], T::par(ui) ^ 1, p.wait_ns);   // the line's previous S is in registers
+        if (!ok) break;
+        tc_fence_after();
+        if (elect_one()) {
 #pragma unroll
           for (int kk = 0; kk < 8; ++kk) {
-            const uint32_t koff16 = (kk >> 2) * (kHalfBytes >> 4) + (kk & 3) * 2;
-            const uint32_t qoff16 = (kk >> 2) * qhalf16 + (kk & 3) * 2;
-            mma_bf16(tmem + 256 + t * 128 + mt * kAttnUnitKeys, dq + qoff16, dk + koff16, idesc_s, kk > 0);
+            const uint64_t b = dk + ((kk >> 2) * (kHalfBytes >> 4) + (kk & 3) * 2);
+            if (kk < T::kTsSteps)
+              mma_f16_ts(tmem + T::s(ln), tmem + T::q(mt) + kk * 8, b, idesc_s, kk > 0);
+            else   // M tile 1: rows 128 on; rows past q_rows feed accumulator rows that no thread reads
+              mma_bf16(tmem + T::s(ln), dq1 + (mt * ((128 * 128) >> 4) + (kk & 3) * 2), b, idesc_s, 1);
           }
-          mma_commit(&ctl->s_full[t][mt]);   // that M tile's softmax starts without waiting for the next
+          mma_commit(&ctl->s_full[ln]);   // that M tile's softmax starts without waiting for the next
+          if (mt == (TWO ? 1 : 0)) mma_commit(&ctl->k_empty[stage]);
+          if (TWO && mt == 1 && i + 1 == c.n) mma_commit(&ctl->q_empty);
         }
-        mma_commit(&ctl->k_empty[stage]);
-        if (i + 1 == c.n) mma_commit(&ctl->q_empty);
+        __syncwarp();
       }
-      __syncwarp();
       if (++stage == p.kv_stages) {
         stage = 0;
         kphase ^= 1;
@@ -319,8 +343,10 @@ __device__ void mma_s_loop(const AttnParams& p, AttnCtl* ctl, const uint8_t* sQ,
   warp_wait(&ctl->drain, 0, drain_limit(p.wait_ns));
 }
 
+template <bool TWO>
 __device__ void mma_pv_loop(const AttnParams& p, AttnCtl* ctl, const uint8_t* sV, uint32_t tmem, int64_t fb,
                             int64_t fe) {
+  using T = Tmem<TWO>;
   const uint32_t idesc_o = idesc_f16_bmn(128, kHeadDim);
   const uint64_t dv0 = sdesc_mn_sw128(smem_u32(sV), kHalfBytes, 1024);
   int stage = 0, vphase = 0;
@@ -329,31 +355,25 @@ __device__ void mma_pv_loop(const AttnParams& p, AttnCtl* ctl, const uint8_t* sV
   for (PieceIter c(p, fb, fe); ok && c.valid(); c.next(p)) {
     ok = !__any_sync(kFull, ctl->abort);
     for (int i = 0; ok && i < c.n; ++i, ++ui) {
-      const int t = static_cast<int>(ui & 1);
       ok = warp_wait(&ctl->v_ready[stage], vphase, p.wait_ns);
       const uint64_t dv = dv0 + static_cast<uint64_t>(stage * (kUnitBytes >> 4));
 #pragma unroll
-      for (int mt = 0; mt < 2; ++mt) {
-        if (mt >= p.n_mtiles || !ok) break;
+      for (int mt = 0; mt < (TWO ? 2 : 1); ++mt) {
         // each M tile's product as soon as its P is written
-        ok = warp_wait(&ctl->p_full[t][mt], (ui >> 1) & 1, p.wait_ns);
+        const int ln = T::line(ui, mt);
+        ok = ok && warp_wait(&ctl->p_full[ln], T::par(ui), p.wait_ns);
         if (!ok) break;
         tc_fence_after();
-        const uint32_t ap = tmem + 256 + t * 128 + mt * kAttnUnitKeys;   // P of M tile mt over its S columns
         if (elect_one()) {
 #pragma unroll
           for (int kk = 0; kk < 4; ++kk)   // 16 keys per step: +8 columns of P, +16 rows of V; the piece's first product overwrites O
-            mma_f16_ts(tmem + mt * kHeadDim, ap + kk * 8, dv + static_cast<uint64_t>(kk * 128), idesc_o,
+            mma_f16_ts(tmem + T::o(mt), tmem + T::p(ln) + kk * 8, dv + static_cast<uint64_t>(kk * 128), idesc_o,
                        (i > 0 || kk > 0) ? 1u : 0u);
+          mma_commit(&ctl->p_empty[ln]);
+          if (mt == (TWO ? 1 : 0)) mma_commit(&ctl->v_empty[stage]);
         }
         __syncwarp();
       }
-      if (!ok) break;
-      if (elect_one()) {
-        mma_commit(&ctl->v_empty[stage]);
-        mma_commit(&ctl->s_empty[t]);   // S stage t (holding P) is free for S two units later
-      }
-      __syncwarp();
       if (++stage == p.kv_stages) {
         stage = 0;
         vphase ^= 1;
@@ -365,7 +385,8 @@ __device__ void mma_pv_loop(const AttnParams& p, AttnCtl* ctl, const uint8_t* sV
   warp_wait(&ctl->drain, 0, drain_limit(p.wait_ns));
 }
 
-// Maximum raw logit of a thread's row over the unit's first `lim` keys.
+// Maximum raw logit of a thread's row over the unit's first `lim` keys (FULL: all 64).
+template <bool FULL>
 __device__ __forceinline__ float unit_max(const uint32_t (&z)[4][16], int lim) {
   float pm[8];   // eight independent partial maxima (short dependency chains)
 #pragma unroll
@@ -374,7 +395,7 @@ __device__ __forceinline__ float unit_max(const uint32_t (&z)[4][16], int lim) {
   for (int q = 0; q < 4; ++q)
 #pragma unroll
     for (int i = 0; i < 16; ++i)
-      if (q * 16 + i < lim) pm[i & 7] = fmaxf(pm[i & 7], __uint_as_float(z[q][i]));
+      if (FULL || q * 16 + i < lim) pm[i & 7] = fmaxf(pm[i & 7], __uint_as_float(z[q][i]));
   return fmaxf(fmaxf(fmaxf(pm[0], pm[1]), fmaxf(pm[2], pm[3])), fmaxf(fmaxf(pm[4], pm[5]), fmaxf(pm[6], pm[7])));
 }
 
@@ -398,38 +419,14 @@ __device__ __forceinline__ void exp_pack_chunk(const uint32_t (&z)[16], int k0, 
 
 // p = exp2(z c2 - m) of the unit's 64 keys (0 past `lim`) as fp16 pairs h[q][j] = (p[16 q + 2 j], p[16 q + 2 j + 1]), the
 // lower key in the low half; returns the sum of the p.
+template <bool FULL>
 __device__ __forceinline__ float exp_pack_p(const uint32_t (&z)[4][16], int lim, float c2, float m,
                                             uint32_t (&h)[4][8]) {
   const float2 sc2 = make_float2(c2, c2), nm2 = make_float2(-m, -m);
   float2 acc[4] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f),
                    make_float2(0.f, 0.f)};   // four independent running sums
 #pragma unroll
-  for (int q = 0; q < 4; ++q) exp_pack_chunk<false>(z[q], 16 * q, lim, sc2, nm2, acc, h[q]);
-  const float2 a01 = fadd2(acc[0], acc[1]), a23 = fadd2(acc[2], acc[3]);
-  const float2 a = fadd2(a01, a23);
-  return a.x + a.y;
-}
-
-// exp_pack_p of a unit of 64 valid keys, reading S itself from `scol` in two halves, the second half's
-// loads in flight under the first half's arithmetic (measured faster than
-// waiting for all four loads first, and than one 16-column load ahead)
-__device__ __forceinline__ float exp_pack_p_streamed(uint32_t scol, float c2, float m, uint32_t (&h)[4][8]) {
-  const float2 sc2 = make_float2(c2, c2), nm2 = make_float2(-m, -m);
-  float2 acc[4] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f),
-                   make_float2(0.f, 0.f)};   // four independent running sums
-  uint32_t a0[16], a1[16], b0[16], b1[16];
-  tmem_ld16_async(scol, a0);
-  tmem_ld16_async(scol + 16, a1);
-  tmem_wait16(a0);
-  tmem_wait16(a1);
-  tmem_ld16_async(scol + 32, b0);
-  tmem_ld16_async(scol + 48, b1);
-  exp_pack_chunk<true>(a0, 0, kAttnUnitKeys, sc2, nm2, acc, h[0]);
-  exp_pack_chunk<true>(a1, 16, kAttnUnitKeys, sc2, nm2, acc, h[1]);
-  tmem_wait16(b0);
-  tmem_wait16(b1);
-  exp_pack_chunk<true>(b0, 32, kAttnUnitKeys, sc2, nm2, acc, h[2]);
-  exp_pack_chunk<true>(b1, 48, kAttnUnitKeys, sc2, nm2, acc, h[3]);
+  for (int q = 0; q < 4; ++q) exp_pack_chunk<FULL>(z[q], 16 * q, lim, sc2, nm2, acc, h[q]);
   const float2 a01 = fadd2(acc[0], acc[1]), a23 = fadd2(acc[2], acc[3]);
   const float2 a = fadd2(a01, a23);
   return a.x + a.y;
@@ -456,102 +453,141 @@ __device__ __forceinline__ void rescale_o(uint32_t o_addr, float alpha) {
   }
 }
 
-// One unit of a softmax warp (warp-uniform `wactive`; TMEM loads and stores
-// are warp-collective): S at `scol` becomes P over its first 32 columns, and
-// the reference m and sum l of the thread's row advance.  `fresh`: the
-// piece's first unit, whose maximum sets the reference.  P is computed with
-// the current reference; every p is below 2^15 unless the unit's sum exceeds
-// it, and only then is the maximum taken (S is still in place, P is stored
-// last): lanes where it lies more than 15 above the reference move it and
-// rescale their O rows (at o_addr, once the product of the previous unit,
-// phase `prev_par` of `prev_bar`, is done), and P is redone.  Returns false
-// when that wait ran out.
-__device__ __forceinline__ bool softmax_unit(const AttnParams& p, bool wactive, bool live, bool fresh, int lim,
-                                             uint32_t scol, uint32_t o_addr, uint64_t* prev_bar, uint32_t prev_par,
-                                             float& m, float& l) {
+// One unit of a softmax warp with rows: S at `scol` into registers, which
+// releases its stage (`s_bar`), then P to `pcol` once the product that read the
+// line's previous P is done (`p_bar`, `p_par`); the reference m and sum l of the
+// thread's row advance.  `fresh`: the piece's first unit, whose maximum sets the
+// reference.  Lanes where a later unit's maximum lies more than 15 above the
+// reference move it and rescale their O rows (at o_addr, once the product of the
+// previous unit, phase `prev_par` of `prev_bar`, is done).  Returns false when a
+// wait ran out.
+template <bool FULL>
+__device__ __forceinline__ bool softmax_unit(const AttnParams& p, int lane, bool live, bool fresh, int lim, uint32_t scol,
+                                             uint64_t* s_bar, uint32_t pcol, uint64_t* p_bar, uint32_t p_par,
+                                             uint32_t o_addr, uint64_t* prev_bar, uint32_t prev_par, float& m,
+                                             float& l) {
   const float c2 = p.scale2;
-  if (fresh) l = 0.f;
-  if (!wactive) {
-    if (fresh) m = 0.f;   // a warp without rows keeps a finite reference
-    return true;
-  }
   uint32_t z[4][16];
   uint32_t h[4][8];
-  float us;
-  if (fresh || lim < kAttnUnitKeys) {
-    load_s(scol, z);
-    if (fresh) m = unit_max(z, lim) * c2;
-    us = exp_pack_p(z, lim, c2, m, h);
+  load_s(scol, z);
+  tc_fence_before();
+  __syncwarp();
+  if (lane == 0) mbar_arrive(s_bar);
+  const float mx = unit_max<FULL>(z, lim) * c2;
+  if (fresh) {
+    m = mx;
+    l = 0.f;
   } else {
-    us = exp_pack_p_streamed(scol, c2, m, h);
-  }
-  if (__any_sync(kFull, live && us > 32768.f)) {   // rare
-    load_s(scol, z);   // z again, so that it need not live across the first pass
-    const float mx = unit_max(z, lim) * c2;
     const bool move = live && mx > m + kMoveThreshold;
-    if (__any_sync(kFull, move)) {
+    if (__any_sync(kFull, move)) {   // rare
       const float alpha = move ? ex2_approx(m - mx) : 1.f;
       if (move) m = mx;
-      if (!__all_sync(kFull, mbar_wait(prev_bar, prev_par, p.wait_ns))) return false;
+      if (!warp_wait(prev_bar, prev_par, p.wait_ns)) return false;
       tc_fence_after();
       rescale_o(o_addr, alpha);
       l *= alpha;
     }
-    // P again in every lane (the same values where the reference stayed), so
-    // that the first h need not live across the reload either
-    us = exp_pack_p(z, lim, c2, m, h);
   }
+  l += exp_pack_p<FULL>(z, lim, c2, m, h);
+  if (!warp_wait(p_bar, p_par, p.wait_ns)) return false;
+  tc_fence_after();
 #pragma unroll
-  for (int q = 0; q < 4; ++q) tmem_st8(scol + q * 8, h[q]);   // keys 16 q ..: columns 8 q ..
-  l += us;
+  for (int q = 0; q < 4; ++q) tmem_st8(pcol + q * 8, h[q]);   // keys 16 q ..: columns 8 q ..
   return true;
 }
 
-constexpr int kSStages = 2;   // S stages in tensor memory
+// This thread's row of a piece's queries, from shared memory ([2 halves][q_rows]
+// [128 B], 16-byte chunks at chunk xor row) to the 64 columns at `dst`.
+template <int HALVES>
+__device__ __forceinline__ void queries_to_tmem(const uint8_t* sQ, int q_rows, int r, bool live, uint32_t dst) {
+#pragma unroll 1
+  for (int h = 0; h < HALVES; ++h) {
+    const uint8_t* row = sQ + (h * q_rows + r) * 128;
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      uint32_t v[16];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const uint4 w = live ? *reinterpret_cast<const uint4*>(row + (((4 * k + i) ^ (r & 7)) << 4))
+                             : make_uint4(0u, 0u, 0u, 0u);
+        v[4 * i] = w.x, v[4 * i + 1] = w.y, v[4 * i + 2] = w.z, v[4 * i + 3] = w.w;
+      }
+      tmem_st16(dst + h * 32 + k * 16, v);
+    }
+  }
+  tmem_wait_st();
+}
 
 // Softmax warps: one thread per window row of M tile `mt` (TMEM lane
-// quad * 32 + lane).  Unit u sits in S stage u mod kSStages; the S (then P)
-// columns of stage t start at s_col0 + t s_stride and O at o_col.  A piece's
-// partial goes to slot row + slot0.
-
-__device__ void softmax_loop(const AttnParams& p, AttnCtl* ctl, uint32_t tmem, int mt, int quad, int lane,
-                             uint32_t s_col0, uint32_t s_stride, uint32_t o_col, int slot0, int64_t fb, int64_t fe) {
-  const int rho = quad * 32 + lane;   // row within the M tile (TMEM lane)
-  const int r = mt * 128 + rho;       // window row within the group
-  if (mt >= p.n_mtiles) return;   // no S is computed for this M tile, no P awaited from it
+// quad * 32 + lane).  A piece's partial goes to slot row + slot0.
+template <bool TWO>
+__device__ void softmax_loop(const AttnParams& p, AttnCtl* ctl, const uint8_t* sQ, uint32_t tmem, int mt, int quad,
+                             int lane, int slot0, int64_t fb, int64_t fe) {
+  using T = Tmem<TWO>;
+  const int r = mt * 128 + quad * 32 + lane;   // window row within the group
   const bool wactive = mt * 128 + quad * 32 < p.rows;
   const bool live = r < p.rows;
   const uint32_t lane_base = tmem + (static_cast<uint32_t>(quad * 32) << 16);
+  const uint32_t o_col = T::o(mt);
   float m = -INFINITY, l = 0.f;
   uint32_t ui = 0;
+  int pc = 0;
+  // the next piece's queries; no product that reads the previous piece's is
+  // left, since this M tile's last S was found ready
+  auto take_queries = [&]() {
+    if (!__all_sync(kFull, mbar_wait(&ctl->q_full, pc & 1, p.wait_ns))) {
+      fail(ctl, p.err);
+      return;
+    }
+    ++pc;
+    if (wactive) queries_to_tmem<T::kTsSteps / 4>(sQ, p.q_rows, r, live, lane_base + T::q(mt));
+    tc_fence_before();
+    __syncwarp();
+    if (lane == 0) {
+      mbar_arrive(&ctl->q_empty);
+      mbar_arrive(&ctl->qt_full);
+    }
+  };
+  if (fb < fe) take_queries();
   for (PieceIter c(p, fb, fe); c.valid() && !ctl->abort; c.next(p)) {
     int lim = p.seq[c.s].Lp - c.j0 * kAttnUnitKeys;   // valid keys from the unit's first on (>= 1)
     for (int i = 0; i < c.n; ++i, ++ui, lim -= kAttnUnitKeys) {
       if (ctl->abort) break;
-      const int t = static_cast<int>(ui % kSStages);
-      const uint32_t par = (ui / kSStages) & 1u;
-      const uint32_t scol = s_col0 + t * s_stride;   // this unit's S, then P, columns
-      if (!__all_sync(kFull, mbar_wait(&ctl->s_full[t][mt], par, p.wait_ns))) {
+      const int ln = T::line(ui, mt);
+      const uint32_t par = T::par(ui);
+      if (!warp_wait(&ctl->s_full[ln], par, p.wait_ns)) {
         fail(ctl, p.err);
         break;
       }
       tc_fence_after();
-      const uint32_t up = ui - 1;   // the previous unit (a piece's first unit never moves)
-      if (!softmax_unit(p, wactive, live, i == 0, lim, lane_base + scol, lane_base + o_col,
-                        &ctl->s_empty[up % kSStages], (up / kSStages) & 1u, m, l)) {
+      bool ok = true;
+      if (wactive) {
+        const uint32_t up = ui - 1;   // the previous unit (a piece's first unit never moves)
+        auto unit = [&](auto full) {
+          return softmax_unit<decltype(full)::value>(p, lane, live, i == 0, lim, lane_base + T::s(ln),
+                                                     &ctl->s_empty[ln], lane_base + T::p(ln), &ctl->p_empty[ln], par ^ 1,
+                                                     lane_base + o_col, &ctl->p_empty[T::line(up, mt)], T::par(up), m, l);
+        };
+        ok = lim >= kAttnUnitKeys ? unit(std::true_type()) : unit(std::false_type());
+      } else {   // a warp without rows only keeps the counts (one phase of each barrier a unit)
+        if (lane == 0) mbar_arrive(&ctl->s_empty[ln]);
+        ok = warp_wait(&ctl->p_empty[ln], par ^ 1, p.wait_ns);
+      }
+      if (!ok) {
         fail(ctl, p.err);
         break;
       }
       tmem_wait_st();
       tc_fence_before();
       __syncwarp();
-      if (lane == 0) mbar_arrive(&ctl->p_full[t][mt]);
+      if (lane == 0) mbar_arrive(&ctl->p_full[ln]);
     }
     if (ctl->abort) break;
+    if (!TWO && c.rem > c.n) take_queries();   // ahead of this piece's partial: S of the next piece runs under it
     // the piece's partial: (m, l) and the unnormalised O rows, once the
     // product of its last unit is done
     const uint32_t lu = ui - 1;
-    if (!__all_sync(kFull, mbar_wait(&ctl->s_empty[lu % kSStages], (lu / kSStages) & 1u, p.wait_ns))) {
+    if (!warp_wait(&ctl->p_empty[T::line(lu, mt)], T::par(lu), p.wait_ns)) {
       fail(ctl, p.err);
       break;
     }
@@ -574,6 +610,7 @@ __device__ void softmax_loop(const AttnParams& p, AttnCtl* ctl, uint32_t tmem, i
       if (live) p.part_ml[slot * kMaxRows + r] = make_float2(m, l);
     }
     tc_fence_before();
+    if (TWO && c.rem > c.n) take_queries();   // (their buffer was free once the piece's last S was done)
   }
 }
 
@@ -611,6 +648,8 @@ __device__ void convert_loop(const AttnParams& p, AttnCtl* ctl, uint8_t* sV, int
 
 }  // namespace
 
+// TWO: the window rows fill two M tiles (more than 128).
+template <bool TWO>
 __global__ void __launch_bounds__(kAttnThreads, 1) k_window_attn(const __grid_constant__ AttnParams p) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -629,14 +668,14 @@ __global__ void __launch_bounds__(kAttnThreads, 1) k_window_attn(const __grid_co
       mbar_init(&ctl->v_ready[i], kConvWarps);
     }
     for (int i = 0; i < 2; ++i) {
-      for (int m = 0; m < 2; ++m) {
-        mbar_init(&ctl->s_full[i][m], 1);
-        mbar_init(&ctl->p_full[i][m], kSoftWarps / 2);   // the four warps of the M tile
-      }
-      mbar_init(&ctl->s_empty[i], 1);   // the P V issuer's commit
+      mbar_init(&ctl->s_full[i], 1);
+      mbar_init(&ctl->s_empty[i], kSoftWarps / 2);   // the four warps of the M tile
+      mbar_init(&ctl->p_full[i], kSoftWarps / 2);
+      mbar_init(&ctl->p_empty[i], 1);                // the P V issuer's commit
     }
     mbar_init(&ctl->q_full, 1);
-    mbar_init(&ctl->q_empty, 1);
+    mbar_init(&ctl->q_empty, TWO ? kSoftWarps + 1 : kSoftWarps / 2);   // (and with two M tiles the S issuer's commit)
+    mbar_init(&ctl->qt_full, TWO ? kSoftWarps : kSoftWarps / 2);
     mbar_init(&ctl->drain, 2);   // one commit per MMA issuer
     ctl->abort = 0;
     fence_mbar_init();
@@ -660,12 +699,12 @@ __global__ void __launch_bounds__(kAttnThreads, 1) k_window_attn(const __grid_co
   } else if (warp == 3) {
     if (lane == 0) v_loader(p, ctl, sV, fb, fe);
   } else if (warp == 1) {
-    mma_s_loop(p, ctl, sQ, sK, tmem, fb, fe);
+    mma_s_loop<TWO>(p, ctl, sQ, sK, tmem, fb, fe);
   } else if (warp == 2) {
-    mma_pv_loop(p, ctl, sV, tmem, fb, fe);
+    mma_pv_loop<TWO>(p, ctl, sV, tmem, fb, fe);
   } else if (warp >= kSoftWarp0 && warp < kSoftWarp0 + kSoftWarps) {
     const int mt = (warp - kSoftWarp0) >> 2;
-    softmax_loop(p, ctl, tmem, mt, warp & 3, lane, 256 + mt * kAttnUnitKeys, 128, mt * kHeadDim, blockIdx.x, fb, fe);
+    if (mt == 0 || TWO) softmax_loop<TWO>(p, ctl, sQ, tmem, mt, warp & 3, lane, blockIdx.x, fb, fe);
   } else if (warp >= kConvWarp0) {
     convert_loop<kConvWarps>(p, ctl, sV, p.kv_stages, threadIdx.x - 32 * kConvWarp0, lane, fb, fe);
   }
@@ -752,8 +791,10 @@ int attn_kv_stages(int q_rows) {
 }
 
 cudaError_t attn_configure() {
-  return cudaFuncSetAttribute(k_window_attn, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              static_cast<int>(kSmemLimit));
+  const int bytes = static_cast<int>(kSmemLimit);
+  const cudaError_t e = cudaFuncSetAttribute(k_window_attn<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  if (e != cudaSuccess) return e;
+  return cudaFuncSetAttribute(k_window_attn<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
 }
 
 namespace {
@@ -777,7 +818,7 @@ cudaError_t attn_main_launch(const AttnParams& p, cudaStream_t stream) {
   if (p.total_units <= 0) return cudaSuccess;
   cudaLaunchAttribute attr[1];
   cudaLaunchConfig_t cfg = pdl_config(attr, dim3(p.grid), dim3(kAttnThreads), attn_smem_bytes(p.q_rows, p.kv_stages), stream);
-  return cudaLaunchKernelEx(&cfg, k_window_attn, p);
+  return cudaLaunchKernelEx(&cfg, p.n_mtiles == 2 ? k_window_attn<true> : k_window_attn<false>, p);
 }
 
 cudaError_t attn_combine_launch(const AttnParams& p, cudaStream_t stream) {
