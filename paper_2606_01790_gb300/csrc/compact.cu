@@ -18,6 +18,11 @@ constexpr int kCompactThreads = 256;
 constexpr int kWarps = kCompactThreads / 32;
 constexpr int kTaskRows = 32;   // output rows per warp task
 constexpr int kInFlight = 8;    // 16-byte accesses per lane in flight (16 rows per warp)
+// 64 registers a thread and four blocks per SM (128 KB of loads in flight).  Left
+// to itself the compiler takes 76 registers, three blocks: 28 layers x 4 heads of
+// 14,032 / 56,128 tokens, 20 % kept, take 50 / 194 us that way and 48 / 185 us so,
+// which is the rate of a plain copy.  Five blocks (51 registers) spill: 56 / 203.
+constexpr int kBlocksPerSm = 4;
 
 __device__ __forceinline__ uint4 ld_stream(const uint4* p) {
   uint4 v;
@@ -37,7 +42,7 @@ __device__ __forceinline__ void st_stream(uint4* p, const uint4& v) {
 
 // grid: (blocks, nlayers, nseq).  Tasks of one (seq, layer): 2 tensors x G x
 // ceil((B + w) / 32) row blocks, one per warp, strided over the grid.
-__global__ void __launch_bounds__(kCompactThreads) k_compact(const __grid_constant__ SeqBatch b, int G, int w,
+__global__ void __launch_bounds__(kCompactThreads, kBlocksPerSm) k_compact(const __grid_constant__ SeqBatch b, int G, int w,
                                                               int per_head, uint32_t* err) {
   griddep_launch_dependents();
   griddep_wait();   // idx comes from the previous kernel
