@@ -335,6 +335,8 @@ SeqView make_view(const starkv_state* st, const starkv_seq& s, char* ws, const W
 }
 
 // Both scoring passes for sequences [i0, i1) over layers [layer0, layer0 + nlayers).
+constexpr int64_t kL2Tiles = 4096;   // 32 KB K tiles in 128 MB of L2
+
 starkv_status run_score(starkv_state* st, const starkv_seq* seqs, int i0, int i1, int layer0, int nlayers,
                         char* ws, const WsPlan& plan, size_t* partial_cursor, cudaStream_t stream) {
   const starkv_config& c = st->cfg;
@@ -385,6 +387,7 @@ starkv_status run_score(starkv_state* st, const starkv_seq* seqs, int i0, int i1
   p.err = st->dev.err;
   p.wait_ns = st->wait_ns;
   p.after_lse = need_lse;
+  p.reverse2 = need_lse && p.n_mtiles == 1 && tiles > kL2Tiles;
   if (need_lse)
     CUDA_TRY(launch(st, STARKV_KERNEL_SCORE_LSE, stream, [&] { return score_lse_launch(p, p.grid1, stream); }));
   CUDA_TRY(launch(st, STARKV_KERNEL_SCORE_ACCUM, stream, [&] { return score_accum_launch(p, p.grid1, stream); }));

@@ -84,10 +84,12 @@ __device__ __forceinline__ TileCoord decode(const ScoreParams& p, int64_t f) {
 
 __device__ __forceinline__ int64_t range_begin(int64_t T, int c, int P) { return T * c / P; }
 
-// The pieces of a CTA's flat range [f0, f1), in order: a piece is a run of n
-// tiles j0, j0 + 1, ... of one (seq, layer, group) row, f its first flat tile.
-// One decode at the start, no divisions after it, and nothing but a counter
-// inside a piece: the tile loops of the four roles carry no coordinates.
+// The pieces of a CTA's flat range [f0, f1), in order (REV: from the last one
+// back): a piece is a run of n tiles j0, j0 + 1, ... of one (seq, layer, group)
+// row, f its first flat tile.  One decode at the start, no divisions after it,
+// and nothing but a counter inside a piece: the tile loops of the four roles
+// carry no coordinates.
+template <bool REV>
 struct PieceIter {
   int s, l, g, j0, n, nt;
   int rem;        // tiles of the range from this piece on
@@ -95,20 +97,37 @@ struct PieceIter {
   __device__ __forceinline__ PieceIter(const ScoreParams& p, int64_t f0, int64_t f1)
       : s(0), l(0), g(0), j0(0), n(0), nt(0), rem(static_cast<int>(f1 - f0)), f(f0) {
     if (rem <= 0) return;
-    const TileCoord c = decode(p, f0);
+    const TileCoord c = decode(p, REV ? f1 - 1 : f0);
     s = c.s;
     l = c.l;
     g = c.g;
-    j0 = c.j;
     nt = p.seq[s].nt;
-    n = min(rem, nt - j0);
+    n = min(rem, REV ? c.j + 1 : nt - c.j);
+    j0 = REV ? c.j + 1 - n : c.j;
+    if (REV) f = f1 - n;
   }
   __device__ __forceinline__ bool valid() const { return rem > 0; }
   __device__ __forceinline__ void next(const ScoreParams& p) {
-    f += n;
     rem -= n;
-    j0 = 0;
+    if (!REV) f += n;
     if (rem <= 0) return;
+    if (REV) {
+      if (--g < 0) {
+        g = p.G - 1;
+        if (--l < 0) {
+          l = p.nlayers - 1;
+          do {
+            --s;
+          } while (s > 0 && p.seq[s].nt == 0);
+          nt = p.seq[s].nt;
+        }
+      }
+      n = min(rem, nt);
+      j0 = nt - n;
+      f -= n;
+      return;
+    }
+    j0 = 0;
     if (++g == p.G) {
       g = 0;
       if (++l == p.nlayers) {
@@ -167,7 +186,7 @@ __device__ __forceinline__ void ctl_init(SmemCtl* ctl, int kstages) {
 // TMA producer shared by both passes.  Q: [2 halves][q_rows][128 B]; pass 1
 // loads the group's rows as a 128-row box and a (rows - 128)-row box per half,
 // pass 2 one n2-row box per half.  K tile: 128 keys as two 64-column halves.
-template <int PASS>
+template <int PASS, bool REV>
 __device__ void producer_loop(const ScoreParams& p, SmemCtl* ctl, uint8_t* sQ, uint8_t* sK,
                               int64_t fb, int64_t fe) {
   const uint64_t pol_k = policy_evict_first();   // K streams through L2 once per pass
@@ -176,7 +195,7 @@ __device__ void producer_loop(const ScoreParams& p, SmemCtl* ctl, uint8_t* sQ, u
   int last_q_pc = -1;
   int last_ph[kMaxStages];
   for (int i = 0; i < kMaxStages; ++i) last_ph[i] = -1;
-  for (PieceIter c(p, fb, fe); c.valid() && !ctl->abort; c.next(p)) {
+  for (PieceIter<REV> c(p, fb, fe); c.valid() && !ctl->abort; c.next(p)) {
     if (!mbar_wait(&ctl->q_empty, (pc & 1) ^ 1, p.wait_ns)) { fail(ctl, p.err); break; }
     const int zq = p.layer0 + c.l, y = c.g * p.rows;
     if (PASS == 1) {
@@ -193,13 +212,17 @@ __device__ void producer_loop(const ScoreParams& p, SmemCtl* ctl, uint8_t* sQ, u
     last_q_pc = pc;
     ++pc;
     const int zk = (p.layer0 + c.l) * p.G + c.g;
-    for (int j = c.j0; j < c.j0 + c.n; ++j) {
+    for (int i = 0; i < c.n; ++i) {
+      const int j = REV ? c.j0 + c.n - 1 - i : c.j0 + i;
       if (ctl->abort) break;
       if (!mbar_wait(&ctl->k_empty[stage], phase ^ 1, p.wait_ns)) { fail(ctl, p.err); break; }
       mbar_arrive_expect_tx(&ctl->k_full[stage], kTileBytes);
       for (int h = 0; h < 2; ++h)
-        tma_load_3d_hint(sK + stage * kTileBytes + h * kHalfBytes, &p.tmk[c.s], &ctl->k_full[stage],
-                         h * 64, j * kTileKeys, zk, pol_k);
+        if (PASS == 1 && p.reverse2)   // what pass 2 reads first is to stay in L2
+          tma_load_3d(sK + stage * kTileBytes + h * kHalfBytes, &p.tmk[c.s], &ctl->k_full[stage], h * 64, j * kTileKeys, zk);
+        else
+          tma_load_3d_hint(sK + stage * kTileBytes + h * kHalfBytes, &p.tmk[c.s], &ctl->k_full[stage], h * 64,
+                           j * kTileKeys, zk, pol_k);
       last_ph[stage] = phase;
       if (++stage == p.kstages) {
         stage = 0;
@@ -222,7 +245,7 @@ __device__ void producer_loop(const ScoreParams& p, SmemCtl* ctl, uint8_t* sQ, u
 // tile.  Issuer `who` owns TMEM accumulator stage `who`; both walk every tile
 // to follow the piece boundaries and each commits the Q release of a piece
 // for its own MMAs.
-template <int PASS>
+template <int PASS, bool REV>
 __device__ void mma_loop(const ScoreParams& p, SmemCtl* ctl, const uint8_t* sQ, const uint8_t* sK,
                          const uint8_t* sX, uint32_t tmem, int64_t fb, int64_t fe, int who) {
   const uint32_t idesc = PASS == 1 ? idesc_bf16(128, kTileKeys) : idesc_bf16(128, p.n2);
@@ -241,7 +264,7 @@ __device__ void mma_loop(const ScoreParams& p, SmemCtl* ctl, const uint8_t* sQ, 
   int stage = who % p.kstages, phase = 0, pc = 0, own = 0;
   const uint32_t d0 = tmem + who * 256;
   int jt = 0;
-  for (PieceIter c(p, fb, fe); c.valid() && !ctl->abort; c.next(p)) {
+  for (PieceIter<REV> c(p, fb, fe); c.valid() && !ctl->abort; c.next(p)) {
     if (!mbar_wait(&ctl->q_full, pc & 1, p.wait_ns)) { fail(ctl, p.err); break; }
     if (PASS == 2) {
       if (!mbar_wait(&ctl->x_full[pc & 1], (pc >> 1) & 1, p.wait_ns)) { fail(ctl, p.err); break; }
@@ -468,9 +491,9 @@ __global__ void __launch_bounds__(kScoreThreads, 1) k_score_lse(const __grid_con
   const int64_t fe = range_begin(T, blockIdx.x + 1, gridDim.x);
 
   if (warp == 0) {
-    if (lane == 0) producer_loop<1>(p, ctl, sQ, sK, fb, fe);
+    if (lane == 0) producer_loop<1, false>(p, ctl, sQ, sK, fb, fe);
   } else if (warp == 1 || warp == 2) {
-    if (lane == 0) mma_loop<1>(p, ctl, sQ, sK, nullptr, tmem, fb, fe, warp - 1);
+    if (lane == 0) mma_loop<1, false>(p, ctl, sQ, sK, nullptr, tmem, fb, fe, warp - 1);
   } else if (warp >= kEpiWarp0) {
     const int wg = (warp - kEpiWarp0) >> 2;  // epilogue warpgroup 0..3
     const int quad = warp & 3;              // TMEM lane quadrant
@@ -489,7 +512,7 @@ __global__ void __launch_bounds__(kScoreThreads, 1) k_score_lse(const __grid_con
     bool dead = false;
     // Every epilogue warp walks every tile and meets the piece-end barrier in
     // the same order; a warp whose wait ran out keeps walking without waiting.
-    for (PieceIter c(p, fb, fe); c.valid(); c.next(p)) {
+    for (PieceIter<false> c(p, fb, fe); c.valid(); c.next(p)) {
       m = -INFINITY;
       s = 0.f;
       int lim = p.seq[c.s].Lp - (c.j0 * kTileKeys + kofs);   // valid keys from this warp's first on
@@ -545,8 +568,9 @@ __global__ void __launch_bounds__(kScoreThreads, 1) k_score_lse(const __grid_con
 // and one row goes to memory instead of four.  A slot is written again at tile
 // j + 8, after every warp has released tile j + 6 and so read the slot before.
 // The piece's last three tiles are stored after a barrier of the epilogue warps.
-// `dst`: this thread's key of the first tile, `left` keys of the row from it on.
-template <int NCH>
+// REV: the tiles go from the piece's last to its first.  `dst`: this thread's key of
+// the first, `left` keys of the row from it on.
+template <int NCH, bool REV>
 __device__ __forceinline__ bool accum_piece(const ScoreParams& p, SmemCtl* ctl, uint32_t base0, float* sS, float* dst, int n,
                                             int left, int jt0, int wg, int q, int quad, int lane, bool dead) {
   const float2 sc2 = make_float2(p.scale2, p.scale2), zero2 = make_float2(0.f, 0.f);
@@ -554,7 +578,8 @@ __device__ __forceinline__ bool accum_piece(const ScoreParams& p, SmemCtl* ctl, 
   auto flush = [&](int i) {   // tile i of the piece, by warpgroup (jt0 + i) mod 4
     if (((jt0 + i) & 3) != wg) return;
     const float* v = sS + ((jt0 + i) & (kSumSlots - 1)) * (4 * kTileKeys) + q;
-    dst[i * kTileKeys] = ((v[0] + v[kTileKeys]) + v[2 * kTileKeys]) + v[3 * kTileKeys];
+    const int key = (REV ? n - 1 - i : i) * kTileKeys;
+    if (key < left) dst[key] = ((v[0] + v[kTileKeys]) + v[2 * kTileKeys]) + v[3 * kTileKeys];
   };
 #pragma unroll 1
   for (int i = 0; i < n; ++i) {
@@ -574,15 +599,24 @@ __device__ __forceinline__ bool accum_piece(const ScoreParams& p, SmemCtl* ctl, 
     __syncwarp();
     if (lane == 0) mbar_arrive(&ctl->t_empty[ts]);
     mine[(jt & (kSumSlots - 1)) * (4 * kTileKeys)] = a.x + a.y;
-    if (i >= 3) flush(i - 3);   // (a whole tile: the row goes on)
+    if (i >= 3) flush(i - 3);
   }
   named_bar_sync(1, kEpiThreads);   // every warp's last sums are written (all reach this, also after a timeout)
   if (!dead)
-    for (int i = max(0, n - 3); i < n; ++i)
-      if (i * kTileKeys < left) flush(i);
+    for (int i = max(0, n - 3); i < n; ++i) flush(i);
   return dead;
 }
 
+// REV: each CTA goes through its range backwards, so that it begins with the K
+// that pass 1 read last and left in L2.  Taken when the launch's K exceeds the L2
+// (below that the order does not matter, and the plain order is 0.3 us faster at
+// one layer of 576 tokens) and one M tile holds the window rows: such passes are
+// bound by HBM.  28 layers of 28 x 14,000 tokens (window 32): 412 -> 380 us,
+// and pass 1, whose K then has no eviction hint, 418 -> 403.  With two M
+// tiles the arithmetic is as long as the K stream: 0.4% faster at best, and pass 1
+// without the hint 4 us slower (14,000 tokens).  Every row's result is the same
+// either way: a key's sum is over the window rows of its own tile.
+template <bool REV>
 __global__ void __launch_bounds__(kScoreThreads, 1) k_score_accum(const __grid_constant__ ScoreParams p) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = align1024(smem_raw);
@@ -614,9 +648,9 @@ __global__ void __launch_bounds__(kScoreThreads, 1) k_score_accum(const __grid_c
   const int64_t fe = range_begin(T, blockIdx.x + 1, gridDim.x);
 
   if (warp == 0) {
-    if (lane == 0) producer_loop<2>(p, ctl, sQ, sK, fb, fe);
+    if (lane == 0) producer_loop<2, REV>(p, ctl, sQ, sK, fb, fe);
   } else if (warp == 1 || warp == 2) {
-    if (lane == 0) mma_loop<2>(p, ctl, sQ, sK, sX, tmem, fb, fe, warp - 1);
+    if (lane == 0) mma_loop<2, REV>(p, ctl, sQ, sK, sX, tmem, fb, fe, warp - 1);
   } else if (warp >= kEpiWarp0) {
     const int et = threadIdx.x - 32 * kEpiWarp0;   // 0..511
     const int wg = et >> 7;                 // column quarter
@@ -633,7 +667,7 @@ __global__ void __launch_bounds__(kScoreThreads, 1) k_score_accum(const __grid_c
     // for a supplied natural-log normaliser) as three bf16 parts (x = hi + mid
     // + lo to about 2^-24 relative) in its K columns 0..2; rows past the
     // group's window rows get a large negative x (exp2 -> 0)
-    auto write_x = [&](const PieceIter& it, int buf) {
+    auto write_x = [&](const PieceIter<REV>& it, int buf) {
       const float* lse = p.seq[it.s].lse;
       float2 part = make_float2(-INFINITY, 0.f);
       if (!lse) {
@@ -677,7 +711,7 @@ __global__ void __launch_bounds__(kScoreThreads, 1) k_score_accum(const __grid_c
       named_bar_sync(1, kEpiThreads);
       if (et == 0) mbar_arrive(&ctl->x_full[buf]);
     };
-    PieceIter c(p, fb, fe);
+    PieceIter<REV> c(p, fb, fe);
     if (c.valid()) {
       // the ones operand: bf16 1.0 in K columns 0..2 of core matrix 0, zeros elsewhere
       if (et < 16) {
@@ -690,7 +724,7 @@ __global__ void __launch_bounds__(kScoreThreads, 1) k_score_accum(const __grid_c
       // the next piece's operand goes to the other buffer now, one piece
       // ahead of its MMAs (this piece's buffer was written one piece earlier;
       // the other one's readers, the previous piece's MMAs, are done)
-      PieceIter nx = c;
+      PieceIter<REV> nx = c;
       nx.next(p);
       if (nx.valid()) write_x(nx, (kp + 1) & 1);
       const ScoreSeq& sq = p.seq[c.s];
@@ -698,11 +732,11 @@ __global__ void __launch_bounds__(kScoreThreads, 1) k_score_accum(const __grid_c
       const int key0 = c.j0 * kTileKeys + q;
       float* dst = sq.s_raw + static_cast<int64_t>(c.l * p.G + c.g) * raw_stride(sq.Lp) + key0;
       switch (nch) {   // this warp's 16-column chunks, the same for the whole launch
-        case 0: dead = accum_piece<0>(p, ctl, base0, sS, dst, c.n, sq.Lp - key0, jt, wg, q, quad, lane, dead); break;
-        case 1: dead = accum_piece<1>(p, ctl, base0, sS, dst, c.n, sq.Lp - key0, jt, wg, q, quad, lane, dead); break;
-        case 2: dead = accum_piece<2>(p, ctl, base0, sS, dst, c.n, sq.Lp - key0, jt, wg, q, quad, lane, dead); break;
-        case 3: dead = accum_piece<3>(p, ctl, base0, sS, dst, c.n, sq.Lp - key0, jt, wg, q, quad, lane, dead); break;
-        default: dead = accum_piece<4>(p, ctl, base0, sS, dst, c.n, sq.Lp - key0, jt, wg, q, quad, lane, dead); break;
+        case 0: dead = accum_piece<0, REV>(p, ctl, base0, sS, dst, c.n, sq.Lp - key0, jt, wg, q, quad, lane, dead); break;
+        case 1: dead = accum_piece<1, REV>(p, ctl, base0, sS, dst, c.n, sq.Lp - key0, jt, wg, q, quad, lane, dead); break;
+        case 2: dead = accum_piece<2, REV>(p, ctl, base0, sS, dst, c.n, sq.Lp - key0, jt, wg, q, quad, lane, dead); break;
+        case 3: dead = accum_piece<3, REV>(p, ctl, base0, sS, dst, c.n, sq.Lp - key0, jt, wg, q, quad, lane, dead); break;
+        default: dead = accum_piece<4, REV>(p, ctl, base0, sS, dst, c.n, sq.Lp - key0, jt, wg, q, quad, lane, dead); break;
       }
       jt += c.n;
       c = nx;
@@ -759,7 +793,9 @@ cudaError_t score_configure() {
   cudaError_t e = cudaFuncSetAttribute(k_score_lse<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(k_score_lse<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
   if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(k_score_accum, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  e = cudaFuncSetAttribute(k_score_accum<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  if (e != cudaSuccess) return e;
+  return cudaFuncSetAttribute(k_score_accum<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
 }
 
 namespace {
@@ -790,7 +826,7 @@ cudaError_t score_lse_launch(const ScoreParams& p, int grid, cudaStream_t stream
 }
 
 cudaError_t score_accum_launch(const ScoreParams& p, int grid, cudaStream_t stream) {
-  return launch_pdl(k_score_accum, dim3(grid), dim3(kScoreThreads), score_smem_bytes(p.q_rows, p.kstages), stream, p);
+  return launch_pdl(p.reverse2 ? k_score_accum<true> : k_score_accum<false>, dim3(grid), dim3(kScoreThreads), score_smem_bytes(p.q_rows, p.kstages), stream, p);
 }
 
 cudaError_t pool_launch(const SeqBatch& b, int G, int H, int pool, int lp_max, cudaStream_t stream) {

@@ -28,6 +28,7 @@ struct ScoreParams {
   int q_rows;          // shared-memory Q rows per 64-column half (= n2)
   int kstages;         // K-tile pipeline depth (from the shared-memory budget)
   int after_lse;       // pass 2 follows this call's pass 1
+  int reverse2;        // pass 2 goes backwards over K that pass 1 left in L2
   int grid1;           // pass-1 grid size (defines the partial-slot partition)
   int64_t total_tiles;
   float scale2;        // log2(e) / sqrt(d)
