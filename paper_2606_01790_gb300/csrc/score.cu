@@ -15,8 +15,10 @@
 //                           operand against the rows' -lse as three bf16
 //                           parts), and each thread sums exp2(acc log2e/sqrt(d))
 //                           over its columns, so the per-key group sum needs
-//                           no cross-lane reduction and no per-column operand.
-//                           The score matrix never leaves the chip.
+//                           no cross-lane reduction and no per-column operand;
+//                           the four column quarters of a key are added on
+//                           chip and one row of sums is stored.  The score
+//                           matrix never leaves the chip.
 // Both passes split the flattened (seq, layer, group, key tile) space into one
 // contiguous range per CTA (persistent grid <= #SMs), so a CTA reloads the
 // group's queries only when its range crosses into a new (seq, layer, group)
@@ -26,8 +28,18 @@
 // exp2 and sums are spread over 16 warps.  Two 256-column TMEM accumulator
 // stages let the MMA of tile i+1 run under the epilogue of tile i; TMEM is
 // read in 16-column loads with the next load in flight under the arithmetic,
-// which runs on packed fp32 pairs.  Each pass is bounded below by its K
-// stream and, at nearly the same level, by the epilogue's per-tile cost.
+// which runs on packed fp32 pairs.
+//
+// What bounds it.  Up to 128 window rows: HBM (28 layers x 28 groups x 14,032
+// tokens: 403 and 380 us for 2.8 GB of K, the rate of a plain copy and above).
+// With two M tiles (224 rows, cycles per tile and SM): pass 1's 16 products take
+// 1,530 at 97 each, where shared memory delivers 8 KB of operands per product;
+// its epilogue's arithmetic 1,175, of which the exp2 unit needs 1,078; the K
+// stream 1,390; in all about 1,690.  Pass 2: 1,230, 1,150 and 1,390.  28 layers x
+// 4 groups x 14,032 tokens: 90 -> 77 us and 72 -> 72 (402 MB; 60 at the copy
+// rate), x 56,128 tokens: 337 -> 287 and 278 -> 271, before -> after the tile
+// loops lost their coordinates, pass 2 its fourfold rows, and pass 2's loads moved
+// under pass 1's tail.
 #include <algorithm>
 #include <utility>
 
@@ -189,7 +201,7 @@ __device__ __forceinline__ void ctl_init(SmemCtl* ctl, int kstages) {
 template <int PASS, bool REV>
 __device__ void producer_loop(const ScoreParams& p, SmemCtl* ctl, uint8_t* sQ, uint8_t* sK,
                               int64_t fb, int64_t fe) {
-  const uint64_t pol_k = policy_evict_first();   // K streams through L2 once per pass
+  const uint64_t pol_k = policy_evict_first();   // K streams through L2 (but see p.reverse2)
   const int qhalf = p.q_rows * 128;
   int stage = 0, phase = 0, pc = 0;
   int last_q_pc = -1;

@@ -48,11 +48,11 @@
 // the loops use has its address taken (the refinement gets its view of the row
 // by value: with closures over the kernel's variables every pass reloaded them
 // from the stack, 40 thousand cycles against 14 in the pooling pass).
-// Measured, one launch, 28 layers unless said: 14,000 tokens 47 -> 35 us (the
-// kernel before: G CTAs of 1024 threads, a row's keys, cells and candidates on
-// chip, whole histograms read from every peer), 56,096 tokens 213 -> 80, the
+// Measured (events), one launch, 28 layers unless said: 14,000 tokens 47 -> 33 us
+// (the kernel before: G CTAs of 1024 threads, a row's keys, cells and candidates
+// on chip, whole histograms read from every peer), 56,096 tokens 213 -> 78, the
 // same 14,000 with 28 groups 268 -> 140, 32 layers of 8 groups x 8,499 tokens
-// 128 -> 40, 16 ragged sequences 917 -> 368, one layer of 568 tokens 32 -> 22.
+// 128 -> 40, 16 ragged sequences 917 -> 366, one layer of 568 tokens 32 -> 21.
 #include <algorithm>
 #include <type_traits>
 
