@@ -207,7 +207,14 @@ __device__ void producer_loop(const ScoreParams& p, SmemCtl* ctl, uint8_t* sQ, u
   int last_q_pc = -1;
   int last_ph[kMaxStages];
   for (int i = 0; i < kMaxStages; ++i) last_ph[i] = -1;
+  // Pass 2 ahead of its dependency wait fills the ring and stops there: a bounded
+  // wait must not run while pass 1 does, whose length has nothing to do with its limit.
+  bool ahead = PASS == 2 && p.after_lse;
   for (PieceIter<REV> c(p, fb, fe); c.valid() && !ctl->abort; c.next(p)) {
+    if (PASS == 2 && ahead && pc > 0) {
+      griddep_wait();
+      ahead = false;
+    }
     if (!mbar_wait(&ctl->q_empty, (pc & 1) ^ 1, p.wait_ns)) { fail(ctl, p.err); break; }
     const int zq = p.layer0 + c.l, y = c.g * p.rows;
     if (PASS == 1) {
@@ -227,6 +234,10 @@ __device__ void producer_loop(const ScoreParams& p, SmemCtl* ctl, uint8_t* sQ, u
     for (int i = 0; i < c.n; ++i) {
       const int j = REV ? c.j0 + c.n - 1 - i : c.j0 + i;
       if (ctl->abort) break;
+      if (PASS == 2 && ahead && phase) {
+        griddep_wait();
+        ahead = false;
+      }
       if (!mbar_wait(&ctl->k_empty[stage], phase ^ 1, p.wait_ns)) { fail(ctl, p.err); break; }
       mbar_arrive_expect_tx(&ctl->k_full[stage], kTileBytes);
       for (int h = 0; h < 2; ++h)
@@ -650,10 +661,11 @@ __global__ void __launch_bounds__(kScoreThreads, 1) k_score_accum(const __grid_c
   __syncthreads();
   tc_fence_after();
   // the set-up above overlaps the previous kernel's tail; its outputs are read
-  // by the epilogue warps.  K and Q are loaded right away when that kernel is
-  // this call's pass 1 (p.after_lse), which waited for whatever wrote them.
+  // by the epilogue warps.  The loader starts on K and Q right away when that
+  // kernel is this call's pass 1 (p.after_lse), which waited for whatever wrote
+  // them; every other role waits for pass 1 here, outside its bounded waits.
   griddep_launch_dependents();
-  if (!p.after_lse || warp >= kEpiWarp0) griddep_wait();
+  if (!p.after_lse || warp != 0) griddep_wait();
   const uint32_t tmem = ctl->tmem_base;
   const int64_t T = p.total_tiles;
   const int64_t fb = range_begin(T, blockIdx.x, gridDim.x);
