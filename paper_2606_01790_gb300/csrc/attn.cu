@@ -512,6 +512,7 @@ __device__ __forceinline__ void queries_to_tmem(const uint8_t* sQ, int q_rows, i
                              : make_uint4(0u, 0u, 0u, 0u);
         v[4 * i] = w.x, v[4 * i + 1] = w.y, v[4 * i + 2] = w.z, v[4 * i + 3] = w.w;
       }
+      __syncwarp();   // (`live` differs between lanes)
       tmem_st16(dst + h * 32 + k * 16, v);
     }
   }
@@ -606,6 +607,7 @@ __device__ void softmax_loop(const AttnParams& p, AttnCtl* ctl, const uint8_t* s
             *reinterpret_cast<float4*>(dst + ch * 16 + i) =
                 make_float4(__uint_as_float(o[i]), __uint_as_float(o[i + 1]), __uint_as_float(o[i + 2]),
                             __uint_as_float(o[i + 3]));
+        __syncwarp();
       }
       if (live) p.part_ml[slot * kMaxRows + r] = make_float2(m, l);
     }

@@ -123,6 +123,7 @@ __device__ __forceinline__ void tmem_relinquish() {
 }
 
 __device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t ncols) {
+  __syncwarp();
   asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols)
                : "memory");
 }
@@ -262,7 +263,11 @@ __device__ __forceinline__ float lg2_approx(float x) {
   return y;
 }
 
+// (the `aligned` instructions of this file want the warp converged; those that
+// follow per-lane branches see to it themselves, since no other rule makes the
+// lanes of a warp meet again before them)
 __device__ __forceinline__ void named_bar_sync(int id, int nthreads) {
+  __syncwarp();
   asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(nthreads) : "memory");
 }
 
@@ -324,6 +329,7 @@ __device__ __forceinline__ uint32_t cluster_rank() {
 // Every thread of every CTA of the cluster; orders shared and global memory
 // accesses before it (release) against those after it (acquire).
 __device__ __forceinline__ void cluster_sync() {
+  __syncwarp();
   asm volatile(
       "barrier.cluster.arrive.release.aligned;\n\t"
       "barrier.cluster.wait.acquire.aligned;" ::: "memory");
@@ -333,9 +339,11 @@ __device__ __forceinline__ void cluster_sync() {
 // every thread arrives after its writes that the peers read, and waits before
 // its first read of a peer's.
 __device__ __forceinline__ void cluster_arrive() {
+  __syncwarp();
   asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
 }
 __device__ __forceinline__ void cluster_wait() {
+  __syncwarp();
   asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 

@@ -442,6 +442,7 @@ __device__ __forceinline__ void lse_tile_slow(uint32_t base, int n, int lim, flo
   const float mn = fmaxf(m, mx * sc);
   if (m != -INFINITY) s *= ex2_approx(m - mn);
   m = mn;
+  __syncwarp();   // (the branch above differs between lanes)
   const float2 sc2 = make_float2(sc, sc), nm2 = make_float2(-m, -m);
   float2 a0 = make_float2(0.f, 0.f), a1 = make_float2(0.f, 0.f);
   for (int ch = 0; ch < n; ++ch) {

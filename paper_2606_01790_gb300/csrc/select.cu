@@ -741,7 +741,6 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_calibrate(const __grid_consta
   // every group's S row, MI_g and phi_g are written: the peers may read them
   // once the barrier completes; the last group's m_g (read by no peer) and the
   // top-B histogram's zeroing go in between
-  __syncwarp();
   cluster_arrive();
   update_m();
   for (int i = tid; i < kBuckets / 4; i += NT) reinterpret_cast<int4*>(hist)[i] = make_int4(0, 0, 0, 0);
@@ -915,10 +914,8 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_calibrate(const __grid_consta
       const int v = __reduce_add_sync(kFullMask, hist[c * kFine + lane]);
       if (lane < r_n) dsmem_st_u32(dsmem_map(reinterpret_cast<int*>(sh.coarse[r_me]) + c, r_lo + lane), static_cast<uint32_t>(v));
     }
-    __syncwarp();
   };
   if (B > 0) send_coarse();
-  __syncwarp();
   cluster_arrive();
   if (per_head) __syncthreads();   // the selection's own exchange; the partial sums are read at the end
   else cluster_wait();
@@ -1071,7 +1068,6 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_calibrate(const __grid_consta
         dsmem_st_u32(dsmem_map(&sh.rlo[r_me], r_lo + lane), sh.lo);
         dsmem_st_u32(dsmem_map(&sh.rhi[r_me], r_lo + lane), sh.hi);
       }
-      __syncwarp();
       if (per_head) __syncthreads();
       else cluster_sync();
       lo = 0xFFFFFFFFu;
@@ -1131,12 +1127,10 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_calibrate(const __grid_consta
       sh.segb[warp] = below;
       if (ties) sh.sege[warp] = eq;
     }
-    __syncwarp();
     const bool wait_peers = !per_head && !ties;
     if (wait_peers) cluster_arrive();
     find_T();   // while the candidates travel
     if (!per_head) write_stats();
-    __syncwarp();
     if (wait_peers) cluster_wait();
     else __syncthreads();
     uint32_t kT = lo, tT = 0u;   // kept: key below kT, or equal to it and (at position <= tT | among the first `quota`)

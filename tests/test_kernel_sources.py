@@ -1,0 +1,38 @@
+"""Rules of the CUDA sources that no run can show to be broken without hanging a GPU:
+read from the text.  CPU only."""
+import re
+from pathlib import Path
+
+import pytest
+
+CSRC = Path(__file__).resolve().parents[1] / "paper_2606_01790_gb300" / "csrc"
+
+
+def functions(name):
+    """{function: body without comments} of the functions of a source file whose
+    brace opens on the line of their closing parenthesis."""
+    text = re.sub(r"//[^\n]*", "", (CSRC / name).read_text())
+    out = {}
+    for m in re.finditer(r"^[^\n;{}=]*?\b(\w+)\((?:[^(){};]|\([^()]*\))*\)\s*\{", text, flags=re.M):
+        if m.group(1) in ("if", "for", "while", "switch"):
+            continue
+        depth, i = 1, m.end()
+        while depth:
+            depth += {"{": 1, "}": -1}.get(text[i], 0)
+            i += 1
+        out[m.group(1)] = text[m.end():i - 1]
+    return out
+
+
+@pytest.mark.parametrize("helper", ["cluster_sync", "cluster_arrive", "cluster_wait", "named_bar_sync", "tmem_dealloc"])
+def test_barriers_that_want_a_converged_warp_converge_it(helper):
+    """An aligned barrier has no time limit: reached by a diverged warp it may
+    never complete.  Callers have per-lane branches right before these."""
+    body = functions("ptx.cuh")[helper]
+    assert "__syncwarp();" in body and body.index("__syncwarp();") < body.index("asm")
+
+
+def test_no_other_source_issues_such_a_barrier_itself():
+    for path in sorted(CSRC.glob("*.cu*")):
+        if path.name != "ptx.cuh":
+            assert not re.search(r'"[^"]*(barrier\.cluster|bar\.sync|tcgen05\.dealloc)', path.read_text()), path.name
