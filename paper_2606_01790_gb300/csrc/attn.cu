@@ -95,6 +95,18 @@ __device__ __forceinline__ void fail(AttnCtl* ctl, uint32_t* err) {
   atomicOr(err, kErrTimeout);
 }
 
+// A wait of a warp-wide role: true when every lane's barrier completed and no
+// role had failed before it.  The one place where these roles learn of a failure,
+// so that a warp's lanes leave together, at the first wait after it (which may
+// itself run for its limit).  `abort` is read ahead of the wait, where it costs
+// nothing (28 layers x 14,000 tokens, 167 us); read behind it the kernel is 4 %
+// slower, read in the sleeping loop 1 %, and a vote ahead of the issuers' waits, which
+// would spare that limit, costs 12 % (once a unit 7 %).
+__device__ __forceinline__ bool warp_wait(const AttnCtl* ctl, uint64_t* bar, uint32_t parity, uint64_t limit_ns) {
+  const bool aborted = ctl->abort;
+  return __all_sync(kFull, mbar_wait(bar, parity, limit_ns) && !aborted);
+}
+
 // Shared-memory descriptor of an MN-major operand in 128-byte swizzled rows
 // (TMA SWIZZLE_128B of a [K][MN] tile, MN contiguous): 64-element MN groups
 // `lbo` bytes apart, 8-row K groups `sbo` bytes apart.
@@ -304,15 +316,15 @@ __device__ void mma_s_loop(const AttnParams& p, AttnCtl* ctl, const uint8_t* sQ,
   uint32_t ui = 0;
   bool ok = true;
   for (PieceIter c(p, fb, fe); ok && c.valid(); c.next(p)) {
-    ok = !__any_sync(kFull, ctl->abort) && warp_wait(&ctl->qt_full, pc & 1, p.wait_ns);
+    ok = warp_wait(ctl, &ctl->qt_full, pc & 1, p.wait_ns);
     ++pc;
     for (int i = 0; ok && i < c.n; ++i, ++ui) {
-      ok = warp_wait(&ctl->k_full[stage], kphase, p.wait_ns);
+      ok = warp_wait(ctl, &ctl->k_full[stage], kphase, p.wait_ns);
       const uint64_t dk = dk0 + static_cast<uint64_t>(stage * (kUnitBytes >> 4));
 #pragma unroll
       for (int mt = 0; mt < (TWO ? 2 : 1); ++mt) {
         const int ln = T::line(ui, mt);
-        ok = ok && warp_wait(&ctl->s_empty[ln], T::par(ui) ^ 1, p.wait_ns);   // the line's previous S is in registers
+        ok = ok && warp_wait(ctl, &ctl->s_empty[ln], T::par(ui) ^ 1, p.wait_ns);   // the line's previous S is in registers
         if (!ok) break;
         tc_fence_after();
         if (elect_one()) {
@@ -340,7 +352,8 @@ __device__ void mma_s_loop(const AttnParams& p, AttnCtl* ctl, const uint8_t* sQ,
   // every MMA issued above must be complete before TMEM is released (the
   // commit tracks the electing lane's: elect_one picks the same lane each time)
   if (elect_one()) mma_commit(&ctl->drain);
-  warp_wait(&ctl->drain, 0, drain_limit(p.wait_ns));
+  mbar_wait(&ctl->drain, 0, drain_limit(p.wait_ns));
+  __syncwarp();
 }
 
 template <bool TWO>
@@ -353,15 +366,14 @@ __device__ void mma_pv_loop(const AttnParams& p, AttnCtl* ctl, const uint8_t* sV
   uint32_t ui = 0;
   bool ok = true;
   for (PieceIter c(p, fb, fe); ok && c.valid(); c.next(p)) {
-    ok = !__any_sync(kFull, ctl->abort);
     for (int i = 0; ok && i < c.n; ++i, ++ui) {
-      ok = warp_wait(&ctl->v_ready[stage], vphase, p.wait_ns);
+      ok = warp_wait(ctl, &ctl->v_ready[stage], vphase, p.wait_ns);
       const uint64_t dv = dv0 + static_cast<uint64_t>(stage * (kUnitBytes >> 4));
 #pragma unroll
       for (int mt = 0; mt < (TWO ? 2 : 1); ++mt) {
         // each M tile's product as soon as its P is written
         const int ln = T::line(ui, mt);
-        ok = ok && warp_wait(&ctl->p_full[ln], T::par(ui), p.wait_ns);
+        ok = ok && warp_wait(ctl, &ctl->p_full[ln], T::par(ui), p.wait_ns);
         if (!ok) break;
         tc_fence_after();
         if (elect_one()) {
@@ -382,7 +394,8 @@ __device__ void mma_pv_loop(const AttnParams& p, AttnCtl* ctl, const uint8_t* sV
   }
   if (!ok) fail(ctl, p.err);
   if (elect_one()) mma_commit(&ctl->drain);
-  warp_wait(&ctl->drain, 0, drain_limit(p.wait_ns));
+  mbar_wait(&ctl->drain, 0, drain_limit(p.wait_ns));
+  __syncwarp();
 }
 
 // Maximum raw logit of a thread's row over the unit's first `lim` keys (FULL: all 64).
@@ -462,10 +475,10 @@ __device__ __forceinline__ void rescale_o(uint32_t o_addr, float alpha) {
 // previous unit, phase `prev_par` of `prev_bar`, is done).  Returns false when a
 // wait ran out.
 template <bool FULL>
-__device__ __forceinline__ bool softmax_unit(const AttnParams& p, int lane, bool live, bool fresh, int lim, uint32_t scol,
-                                             uint64_t* s_bar, uint32_t pcol, uint64_t* p_bar, uint32_t p_par,
-                                             uint32_t o_addr, uint64_t* prev_bar, uint32_t prev_par, float& m,
-                                             float& l) {
+__device__ __forceinline__ bool softmax_unit(const AttnParams& p, const AttnCtl* ctl, int lane, bool live, bool fresh,
+                                             int lim, uint32_t scol, uint64_t* s_bar, uint32_t pcol, uint64_t* p_bar,
+                                             uint32_t p_par, uint32_t o_addr, uint64_t* prev_bar, uint32_t prev_par,
+                                             float& m, float& l) {
   const float c2 = p.scale2;
   uint32_t z[4][16];
   uint32_t h[4][8];
@@ -482,14 +495,14 @@ __device__ __forceinline__ bool softmax_unit(const AttnParams& p, int lane, bool
     if (__any_sync(kFull, move)) {   // rare
       const float alpha = move ? ex2_approx(m - mx) : 1.f;
       if (move) m = mx;
-      if (!warp_wait(prev_bar, prev_par, p.wait_ns)) return false;
+      if (!warp_wait(ctl, prev_bar, prev_par, p.wait_ns)) return false;
       tc_fence_after();
       rescale_o(o_addr, alpha);
       l *= alpha;
     }
   }
   l += exp_pack_p<FULL>(z, lim, c2, m, h);
-  if (!warp_wait(p_bar, p_par, p.wait_ns)) return false;
+  if (!warp_wait(ctl, p_bar, p_par, p.wait_ns)) return false;
   tc_fence_after();
 #pragma unroll
   for (int q = 0; q < 4; ++q) tmem_st8(pcol + q * 8, h[q]);   // keys 16 q ..: columns 8 q ..
@@ -536,10 +549,7 @@ __device__ void softmax_loop(const AttnParams& p, AttnCtl* ctl, const uint8_t* s
   // the next piece's queries; no product that reads the previous piece's is
   // left, since this M tile's last S was found ready
   auto take_queries = [&]() {
-    if (!__all_sync(kFull, mbar_wait(&ctl->q_full, pc & 1, p.wait_ns))) {
-      fail(ctl, p.err);
-      return;
-    }
+    if (!warp_wait(ctl, &ctl->q_full, pc & 1, p.wait_ns)) return false;
     ++pc;
     if (wactive) queries_to_tmem<T::kTsSteps / 4>(sQ, p.q_rows, r, live, lane_base + T::q(mt));
     tc_fence_before();
@@ -548,50 +558,41 @@ __device__ void softmax_loop(const AttnParams& p, AttnCtl* ctl, const uint8_t* s
       mbar_arrive(&ctl->q_empty);
       mbar_arrive(&ctl->qt_full);
     }
+    return true;
   };
-  if (fb < fe) take_queries();
-  for (PieceIter c(p, fb, fe); c.valid() && !ctl->abort; c.next(p)) {
+  bool ok = fb >= fe || take_queries();
+  for (PieceIter c(p, fb, fe); ok && c.valid(); c.next(p)) {
     int lim = p.seq[c.s].Lp - c.j0 * kAttnUnitKeys;   // valid keys from the unit's first on (>= 1)
-    for (int i = 0; i < c.n; ++i, ++ui, lim -= kAttnUnitKeys) {
-      if (ctl->abort) break;
+    for (int i = 0; ok && i < c.n; ++i, ++ui, lim -= kAttnUnitKeys) {
       const int ln = T::line(ui, mt);
       const uint32_t par = T::par(ui);
-      if (!warp_wait(&ctl->s_full[ln], par, p.wait_ns)) {
-        fail(ctl, p.err);
-        break;
-      }
+      ok = warp_wait(ctl, &ctl->s_full[ln], par, p.wait_ns);
+      if (!ok) break;
       tc_fence_after();
-      bool ok = true;
       if (wactive) {
         const uint32_t up = ui - 1;   // the previous unit (a piece's first unit never moves)
         auto unit = [&](auto full) {
-          return softmax_unit<decltype(full)::value>(p, lane, live, i == 0, lim, lane_base + T::s(ln),
+          return softmax_unit<decltype(full)::value>(p, ctl, lane, live, i == 0, lim, lane_base + T::s(ln),
                                                      &ctl->s_empty[ln], lane_base + T::p(ln), &ctl->p_empty[ln], par ^ 1,
                                                      lane_base + o_col, &ctl->p_empty[T::line(up, mt)], T::par(up), m, l);
         };
         ok = lim >= kAttnUnitKeys ? unit(std::true_type()) : unit(std::false_type());
       } else {   // a warp without rows only keeps the counts (one phase of each barrier a unit)
         if (lane == 0) mbar_arrive(&ctl->s_empty[ln]);
-        ok = warp_wait(&ctl->p_empty[ln], par ^ 1, p.wait_ns);
+        ok = warp_wait(ctl, &ctl->p_empty[ln], par ^ 1, p.wait_ns);
       }
-      if (!ok) {
-        fail(ctl, p.err);
-        break;
-      }
+      if (!ok) break;
       tmem_wait_st();
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(&ctl->p_full[ln]);
     }
-    if (ctl->abort) break;
-    if (!TWO && c.rem > c.n) take_queries();   // ahead of this piece's partial: S of the next piece runs under it
+    if (!TWO && ok && c.rem > c.n) ok = take_queries();   // ahead of this piece's partial: S of the next piece runs under it
     // the piece's partial: (m, l) and the unnormalised O rows, once the
     // product of its last unit is done
     const uint32_t lu = ui - 1;
-    if (!warp_wait(&ctl->p_empty[T::line(lu, mt)], T::par(lu), p.wait_ns)) {
-      fail(ctl, p.err);
-      break;
-    }
+    ok = ok && warp_wait(ctl, &ctl->p_empty[T::line(lu, mt)], T::par(lu), p.wait_ns);
+    if (!ok) break;
     tc_fence_after();
     const int64_t slot = static_cast<int64_t>(c.row(p)) + slot0;
     if (wactive) {
@@ -612,8 +613,9 @@ __device__ void softmax_loop(const AttnParams& p, AttnCtl* ctl, const uint8_t* s
       if (live) p.part_ml[slot * kMaxRows + r] = make_float2(m, l);
     }
     tc_fence_before();
-    if (TWO && c.rem > c.n) take_queries();   // (their buffer was free once the piece's last S was done)
+    if (TWO && c.rem > c.n) ok = take_queries();   // (their buffer was free once the piece's last S was done)
   }
+  if (!ok) fail(ctl, p.err);
 }
 
 // V conversion warps (NW of them, thread ct of 32 NW): V of every unit to
@@ -623,8 +625,7 @@ __device__ void convert_loop(const AttnParams& p, AttnCtl* ctl, uint8_t* sV, int
                              int64_t fe) {
   int stage = 0, phase = 0;
   for (int n = static_cast<int>(fe - fb); n > 0; --n) {
-    if (ctl->abort) break;
-    if (!__all_sync(kFull, mbar_wait(&ctl->v_full[stage], phase, p.wait_ns))) {
+    if (!warp_wait(ctl, &ctl->v_full[stage], phase, p.wait_ns)) {
       fail(ctl, p.err);
       break;
     }

@@ -76,11 +76,6 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, uint64
   }
 }
 
-// mbar_wait by a whole warp: true when every lane's succeeded.
-__device__ __forceinline__ bool warp_wait(uint64_t* bar, uint32_t parity, uint64_t limit_ns) {
-  return __all_sync(0xffffffffu, mbar_wait(bar, parity, limit_ns));
-}
-
 // ------------------------------------------------------------------ TMA
 
 // 3-D tiled load into shared memory, completion signalled on `bar` (tx bytes).

@@ -36,3 +36,20 @@ def test_no_other_source_issues_such_a_barrier_itself():
     for path in sorted(CSRC.glob("*.cu*")):
         if path.name != "ptx.cuh":
             assert not re.search(r'"[^"]*(barrier\.cluster|bar\.sync|tcgen05\.dealloc)', path.read_text()), path.name
+
+
+@pytest.mark.parametrize("role", ["mma_s_loop", "mma_pv_loop", "softmax_unit", "softmax_loop", "convert_loop"])
+def test_warp_wide_attention_roles_leave_together(role):
+    """Lanes that read another role's failure flag one by one may disagree, and those
+    that stay then wait for the others in the next warp vote for ever.  These
+    roles learn of a failure only through warp_wait's vote, at every wait; the
+    final wait for their own products is the one that goes on regardless."""
+    body = functions("attn.cu")[role]
+    assert "abort" not in body
+    assert "warp_wait(" in body
+    assert re.findall(r"\bmbar_wait\(([^,]*),", body) == (["&ctl->drain"] if role.startswith("mma") else [])
+
+
+def test_every_attention_wait_sees_another_roles_failure():
+    body = functions("attn.cu")["warp_wait"]
+    assert body.index("ctl->abort") < body.index("__all_sync(") < body.index("mbar_wait(")
