@@ -250,11 +250,11 @@ __device__ void k_loader(const AttnParams& p, AttnCtl* ctl, uint8_t* sQ, uint8_t
       }
     }
   }
-  if (ctl->abort) {   // every issued copy completes before the CTA can exit
-    for (int i = 0; i < kStages; ++i)
-      if (last_ph[i] >= 0) mbar_wait(&ctl->k_full[i], last_ph[i], drain_limit(p.wait_ns));
-    if (last_q_pc >= 0) mbar_wait(&ctl->q_full, last_q_pc & 1, drain_limit(p.wait_ns));
-  }
+  // every issued copy completes before the CTA can exit (also when no wait of this
+  // role ran out: another role may give up after its last load)
+  for (int i = 0; i < kStages; ++i)
+    if (last_ph[i] >= 0) mbar_wait(&ctl->k_full[i], last_ph[i], drain_limit(p.wait_ns));
+  if (last_q_pc >= 0) mbar_wait(&ctl->q_full, last_q_pc & 1, drain_limit(p.wait_ns));
 }
 
 // V loader: a V stage is free once the P V product of its unit is done.
@@ -279,9 +279,8 @@ __device__ void v_loader(const AttnParams& p, AttnCtl* ctl, uint8_t* sV, int64_t
       }
     }
   }
-  if (ctl->abort)
-    for (int i = 0; i < kStages; ++i)
-      if (last_ph[i] >= 0) mbar_wait(&ctl->v_full[i], last_ph[i], drain_limit(p.wait_ns));
+  for (int i = 0; i < kStages; ++i)
+    if (last_ph[i] >= 0) mbar_wait(&ctl->v_full[i], last_ph[i], drain_limit(p.wait_ns));
 }
 
 // A line is what a softmax warpgroup works through in order: with two M tiles

@@ -253,12 +253,11 @@ __device__ void producer_loop(const ScoreParams& p, SmemCtl* ctl, uint8_t* sQ, u
       }
     }
   }
-  if (ctl->abort) {
-    // bring every issued copy to completion before the CTA can exit
-    for (int i = 0; i < p.kstages; ++i)
-      if (last_ph[i] >= 0) mbar_wait(&ctl->k_full[i], last_ph[i], drain_limit(p.wait_ns));
-    if (last_q_pc >= 0) mbar_wait(&ctl->q_full, last_q_pc & 1, drain_limit(p.wait_ns));
-  }
+  // bring every issued copy to completion before the CTA can exit (also when no
+  // wait of this role ran out: another role may give up after its last load)
+  for (int i = 0; i < p.kstages; ++i)
+    if (last_ph[i] >= 0) mbar_wait(&ctl->k_full[i], last_ph[i], drain_limit(p.wait_ns));
+  if (last_q_pc >= 0) mbar_wait(&ctl->q_full, last_q_pc & 1, drain_limit(p.wait_ns));
 }
 
 // MMA issuer shared by both passes.  Two issuing threads (warps 1 and 2)

@@ -53,3 +53,18 @@ def test_warp_wide_attention_roles_leave_together(role):
 def test_every_attention_wait_sees_another_roles_failure():
     body = functions("attn.cu")["warp_wait"]
     assert body.index("ctl->abort") < body.index("__all_sync(") < body.index("mbar_wait(")
+
+
+@pytest.mark.parametrize("source,role", [("score.cu", "producer_loop"), ("attn.cu", "k_loader"), ("attn.cu", "v_loader")])
+def test_loaders_see_every_copy_land(source, role):
+    """A loader that is past its last load when another role gives up still keeps
+    the block until its copies are in: they would land in another block's shared
+    memory.  The waits for them stand at the function's top level."""
+    body = functions(source)[role]
+    depth, found = 0, []
+    for line in body.split("\n"):
+        if "drain_limit(" in line:
+            found.append((depth, line))
+        depth += line.count("{") - line.count("}")
+    assert found and all(d == 0 for d, _ in found)
+    assert not re.search(r"if \(ctl->abort\)\s*\{?\s*for", body)
