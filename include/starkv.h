@@ -385,6 +385,11 @@ starkv_status starkv_set_timing(starkv_state* st, int32_t on);
  * off too (total_ms then stays 0).  Either array may be NULL. */
 starkv_status starkv_kernel_times(starkv_state* st, int64_t* launches, float* total_ms);
 
+/* Launches of scoring pass 2 that went through their tiles backwards, since the
+ * state's creation (taken when the window rows of a group are at most 128 and the
+ * launch's K exceeds the device's L2; the results are the same either way). */
+starkv_status starkv_backward_launches(const starkv_state* st, int64_t* launches);
+
 /* Thread-local message describing the last non-OK status on this thread. */
 const char* starkv_last_error(void);
 

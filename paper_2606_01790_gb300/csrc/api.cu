@@ -29,6 +29,8 @@ struct starkv_state {
   size_t mem_bytes = 0;
   int device = 0;
   int num_sms = 0;
+  int l2_bytes = 0;
+  int64_t backward = 0;   // scoring launches whose pass 2 went backwards
   uint64_t wait_ns = 1000000000ull;
   // kernel timing (starkv_set_timing / starkv_kernel_times)
   bool timing = false;
@@ -335,8 +337,6 @@ SeqView make_view(const starkv_state* st, const starkv_seq& s, char* ws, const W
 }
 
 // Both scoring passes for sequences [i0, i1) over layers [layer0, layer0 + nlayers).
-constexpr int64_t kL2Tiles = 4096;   // 32 KB K tiles in 128 MB of L2
-
 starkv_status run_score(starkv_state* st, const starkv_seq* seqs, int i0, int i1, int layer0, int nlayers,
                         char* ws, const WsPlan& plan, size_t* partial_cursor, cudaStream_t stream) {
   const starkv_config& c = st->cfg;
@@ -387,7 +387,9 @@ starkv_status run_score(starkv_state* st, const starkv_seq* seqs, int i0, int i1
   p.err = st->dev.err;
   p.wait_ns = st->wait_ns;
   p.after_lse = need_lse;
-  p.reverse2 = need_lse && p.n_mtiles == 1 && tiles > kL2Tiles;
+  // one M tile and more K than the L2 holds (k_score_accum gives the reason)
+  p.reverse2 = need_lse && p.n_mtiles == 1 && tiles * (kTileKeys * kHeadDim * 2) > st->l2_bytes;
+  st->backward += p.reverse2;
   if (need_lse)
     CUDA_TRY(launch(st, STARKV_KERNEL_SCORE_LSE, stream, [&] { return score_lse_launch(p, p.grid1, stream); }));
   CUDA_TRY(launch(st, STARKV_KERNEL_SCORE_ACCUM, stream, [&] { return score_accum_launch(p, p.grid1, stream); }));
@@ -618,6 +620,7 @@ starkv_status starkv_init_state(const starkv_config* cfg, starkv_state** out, vo
   st->cfg = *cfg;
   cudaError_t e = cudaGetDevice(&st->device);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&st->num_sms, cudaDevAttrMultiProcessorCount, st->device);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&st->l2_bytes, cudaDevAttrL2CacheSize, st->device);
   if (e == cudaSuccess) e = score_configure();
   if (e == cudaSuccess) e = select_configure();
   if (e == cudaSuccess) e = attn_configure();
@@ -1057,6 +1060,12 @@ starkv_status starkv_kernel_times(starkv_state* st, int64_t* launches, float* to
     st->launches[k] = 0;
   }
   return status;
+}
+
+starkv_status starkv_backward_launches(const starkv_state* st, int64_t* launches) {
+  if (!st || !launches) return set_error(STARKV_ERR_INVALID_ARG, "a pointer is NULL");
+  *launches = st->backward;
+  return STARKV_OK;
 }
 
 const char* starkv_last_error(void) { return g_last_error.c_str(); }

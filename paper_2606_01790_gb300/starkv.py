@@ -25,7 +25,8 @@ ABI_FUNCTIONS = [
     "starkv_default_config", "starkv_init_state", "starkv_reset_seq", "starkv_destroy_state",
     "starkv_get_config", "starkv_workspace_bytes", "starkv_score_layer", "starkv_select",
     "starkv_compact", "starkv_step", "starkv_step_host", "starkv_check_device_error",
-    "starkv_set_wait_limit", "starkv_set_timing", "starkv_kernel_times", "starkv_last_error",
+    "starkv_set_wait_limit", "starkv_set_timing", "starkv_kernel_times", "starkv_backward_launches",
+    "starkv_last_error",
     "starkv_score_layer_noalloc", "starkv_selftest_wait", "starkv_slot_state_bytes", "starkv_export_slot",
     "starkv_import_slot", "starkv_window_attention",
 ]
@@ -110,6 +111,7 @@ def lib() -> C.CDLL:
         L.starkv_import_slot.argtypes = [st, C.c_int32, C.c_void_p, C.c_size_t, C.c_void_p]
         L.starkv_set_timing.argtypes = [st, C.c_int32]
         L.starkv_kernel_times.argtypes = [st, C.POINTER(C.c_int64), C.POINTER(C.c_float)]
+        L.starkv_backward_launches.argtypes = [st, C.POINTER(C.c_int64)]
         L.starkv_last_error.argtypes = []
         L.starkv_last_error.restype = C.c_char_p
         for name in ABI_FUNCTIONS:
@@ -424,3 +426,10 @@ def kernel_times(st: State):
     ms = (C.c_float * n)()
     _check(lib().starkv_kernel_times(st.handle, launches, ms))
     return {k: (int(launches[i]), float(ms[i])) for i, k in enumerate(KERNELS)}
+
+
+def backward_launches(st: State) -> int:
+    """Launches of scoring pass 2 that went through their tiles backwards, so far."""
+    n = C.c_int64(0)
+    _check(lib().starkv_backward_launches(st.handle, C.byref(n)))
+    return int(n.value)

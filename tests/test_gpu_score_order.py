@@ -1,26 +1,29 @@
 """Scoring pass 2 over the tiles in reverse order: taken when one M tile holds
-the window rows and the launch's K exceeds the L2 (more than 4096 128-key tiles).
-Sizes around that line, with ragged last tiles and sequences of one tile between
-long ones, so that a CTA's range ends and begins inside rows.  S of the whole
-step against the softmax sums in 64 bits (Eqs. 2-4) to 1e-5, and against the
-per-layer calls, whose launches are below the line, to 2e-6: the two differ
-only in where the normalisers' partial sums are cut, a few units of 2^-24 each.
+the window rows and the launch's K exceeds the device's L2.  Sizes on both sides of
+that line, with ragged last tiles and sequences of one tile between long ones, so
+that a CTA's range ends and begins inside rows; every number of 16-column chunks
+a warp can hold there; and a row spread over more than eight CTAs, whose normalisers
+two threads merge.  The state's counter shows which order ran.
+
+S of the whole step against the softmax sums in 64 bits (Eqs. 2-4) to 1e-5, and
+against the per-layer calls, whose launches are below the line, to 2e-6: the two
+differ only in where the normalisers' partial sums are cut, a few units of 2^-24
+each.
 """
-import dataclasses
 import math
 
 import pytest
 import torch
 
 from paper_2606_01790_gb300 import starkv as sk
-from paper_2606_01790_gb300 import synthetic as syn
-
-import harness as H
 
 pytestmark = pytest.mark.gpu
 
 if not torch.cuda.is_available():
     pytest.skip("needs a CUDA device", allow_module_level=True)
+
+D = 128
+TILE = 128   # keys
 
 
 @pytest.fixture(scope="module", autouse=True)
@@ -39,21 +42,41 @@ def _reference(q, k, w, pool):
     return a * G / q.shape[0]
 
 
-@pytest.mark.parametrize("texts", [[16399, 30, 16100], [16399, 30, 17, 16100]], ids=["at_the_line", "above"])
-def test_pass_2_backwards(texts):
-    w, G, nl = 8, 4, 4
-    base = dataclasses.replace(syn.WORKLOADS["tiny"], n_heads=8, n_kv_heads=G, window=w, n_layers=nl)
-    tiles = nl * G * sum((t - w + 127) // 128 for t in texts)
-    assert tiles == (4096 if len(texts) == 3 else 4112)
-    hyper = H.hyper()
-    sts = [sk.init_state(H.gpu_config(base, hyper, max_seqs=len(texts))) for _ in range(2)]
-    runs, sis = [], []
-    for i, text in enumerate(texts):
-        wl = dataclasses.replace(base, name=f"o{i}", cfg_id=400 + i, n_shots=0, n_text=text)
-        si = syn.make_sequence(wl)
-        sis.append(si)
-        runs.append([H.device_seq(si, wl, slot=i) for _ in range(2)])
-    whole, layered = ([r[j].seq for r in runs] for j in range(2))
+# heads, groups, window, layers, tiles of the short sequences between the long ones
+SHAPES = [(8, 4, 8, 4, [1]),       # 16 window rows: chunks 1, 0, 0, 0 of the four warpgroups
+          (8, 4, 8, 4, [1, 1]),
+          (12, 4, 31, 4, [3]),     # 93 rows: 2, 2, 1, 1
+          (16, 4, 32, 4, [1]),     # 128 rows: 2, 2, 2, 2
+          (4, 1, 8, 4, [])]        # one sequence: rows of 40 CTAs
+
+
+@pytest.mark.parametrize("above", [False, True], ids=["at_the_line", "above"])
+@pytest.mark.parametrize("heads,G,w,nl,short", SHAPES)
+def test_pass_2_backwards(heads, G, w, nl, short, above):
+    line = torch.cuda.get_device_properties(0).L2_cache_size // (TILE * D * 2)   # tiles that fit
+    n = line // (nl * G) + above - sum(short)    # of the long sequences, per row
+    lens = ([n // 2 * TILE - 17] + [t * TILE - 106 for t in short] + [(n - n // 2) * TILE - 28]) if short else [n * TILE - 5]
+    tiles = nl * G * sum(-(-lp // TILE) for lp in lens)
+    assert (tiles > line) == above and abs(tiles - line) <= nl * G
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(heads + above)
+
+    def normal(*shape):
+        return torch.randn(*shape, generator=gen, device="cuda").to(torch.bfloat16)
+
+    def room(lp):
+        return dict(k_out=torch.empty(nl, G, 1 + w, D, dtype=torch.bfloat16, device="cuda"),
+                    v_out=torch.empty(nl, G, 1 + w, D, dtype=torch.bfloat16, device="cuda"),
+                    meta_out=torch.empty(nl, 1 + w, dtype=torch.int32, device="cuda"),
+                    idx=torch.empty(nl, 1, dtype=torch.int32, device="cuda"), S=torch.empty(nl, G, lp, device="cuda"))
+
+    whole, layered = [], []
+    for i, lp in enumerate(lens):
+        k, q = normal(nl, G, lp + w, D), normal(nl, heads, w, D)
+        meta = torch.zeros(lp + w, dtype=torch.int32, device="cuda")
+        for seqs in (whole, layered):
+            seqs.append(sk.Seq(k=k, v=k, q=q, meta=meta, L=lp + w, budget=1, slot=i, **room(lp)))
+    sts = [sk.init_state(sk.Config(n_layers=nl, n_heads=heads, n_kv_heads=G, window=w, max_seqs=len(lens))) for _ in range(2)]
     sk.step(sts[0], whole, sk.workspace(sts[0], whole))
     ws = sk.workspace(sts[1], layered)
     for layer in range(nl):
@@ -61,15 +84,12 @@ def test_pass_2_backwards(texts):
     torch.cuda.synchronize()
     for st in sts:
         sk.check_device_error(st)
-    for si, a, b in zip(sis, whole, layered):
-        if si.L == w:
-            continue
-        lp = si.L - w
+    assert [sk.backward_launches(st) for st in sts] == [int(above), 0]
+    for a, b in zip(whole, layered):
         for layer in range(nl):
-            got = a.S.reshape(nl, G, lp)[layer].double()
-            ref = _reference(si.q[layer].cuda(), si.k[layer].cuda(), w, 5)
+            got, other = a.S[layer].double(), b.S[layer].double()
+            ref = _reference(a.q[layer], a.k[layer], w, 5)
             assert ((got - ref).abs() / ref.clamp_min(1e-30)).max().item() <= 1e-5
-            other = b.S.reshape(nl, G, lp)[layer].double()
             assert ((got - other).abs() / other.clamp_min(1e-30)).max().item() <= 2e-6
     for st in sts:
         st.close()
