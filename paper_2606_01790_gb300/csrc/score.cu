@@ -289,6 +289,7 @@ __device__ void mma_loop(const ScoreParams& p, SmemCtl* ctl, const uint8_t* sQ, 
   for (PieceIter<REV> c(p, fb, fe); c.valid() && !ctl->abort; c.next(p)) {
     if (!mbar_wait(&ctl->q_full, pc & 1, p.wait_ns)) { fail(ctl, p.err); break; }
     if (PASS == 2) {
+      if (p.after_lse && pc == 0) griddep_wait();   // (as the loader: outside the bounded wait)
       if (!mbar_wait(&ctl->x_full[pc & 1], (pc >> 1) & 1, p.wait_ns)) { fail(ctl, p.err); break; }
       dbx = dbx0 + static_cast<uint64_t>((pc & 1) * ((p.q_rows * kXRowBytes) >> 4));
     }
@@ -661,11 +662,10 @@ __global__ void __launch_bounds__(kScoreThreads, 1) k_score_accum(const __grid_c
   __syncthreads();
   tc_fence_after();
   // the set-up above overlaps the previous kernel's tail; its outputs are read
-  // by the epilogue warps.  The loader starts on K and Q right away when that
-  // kernel is this call's pass 1 (p.after_lse), which waited for whatever wrote
-  // them; every other role waits for pass 1 here, outside its bounded waits.
+  // by the epilogue warps.  K and Q are loaded right away when that kernel is
+  // this call's pass 1 (p.after_lse), which waited for whatever wrote them.
   griddep_launch_dependents();
-  if (!p.after_lse || warp != 0) griddep_wait();
+  if (!p.after_lse || warp >= kEpiWarp0) griddep_wait();
   const uint32_t tmem = ctl->tmem_base;
   const int64_t T = p.total_tiles;
   const int64_t fb = range_begin(T, blockIdx.x, gridDim.x);
