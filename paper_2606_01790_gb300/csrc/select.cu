@@ -182,10 +182,13 @@ constexpr size_t kCalSharedBytes = align16(sizeof(CalShared));
 constexpr int kBucketTable = kBuckets;   // bytes: rank bin of each bucket, or 0x80 | slot
 constexpr int kCandBytes = kCandMax * 8;
 
-size_t fixed_bytes(int K, int M, int R, int C) {
-  return kCalSharedBytes + static_cast<size_t>(kBuckets) * 4 + kCandBytes + align16(static_cast<size_t>(K) * M * M * 4) +
-         align16(static_cast<size_t>(R) * C * 4) + kBucketTable;
+constexpr size_t fixed_bytes(int joint_cells, int patches) {   // K M^2, R C
+  return kCalSharedBytes + static_cast<size_t>(kBuckets) * 4 + kCandBytes + align16(static_cast<size_t>(joint_cells) * 4) +
+         align16(static_cast<size_t>(patches) * 4) + kBucketTable;
 }
+// Two CTAs without a row on chip fit an SM whatever the configuration (228 KB, of
+// which each takes 1 KB more): the two-per-SM variant never runs alone.
+static_assert(fixed_bytes(kMaxHist, kMaxGrid) + 1024 <= 114 * 1024, "two CTAs fit");
 
 constexpr size_t kBytesPerToken = 4;   // a row's keys, then the CTA's fused scores
 
@@ -1208,8 +1211,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_calibrate(const __grid_consta
 
 namespace {
 
-int calibrate_capacity(int K, int M, int R, int C, size_t smem) {
-  const size_t fixed = fixed_bytes(K, M, R, C);
+int calibrate_capacity(size_t fixed, size_t smem) {
   if (fixed >= smem) return 0;
   return static_cast<int>(((smem - fixed) / kBytesPerToken) & ~size_t(15));
 }
@@ -1239,14 +1241,18 @@ cudaError_t calibrate_launch(const SeqBatch& b, const KParams& kp, const DevStat
   // More CTAs than SMs: 512 threads and at most half of the shared memory
   // each, so that two run on an SM and one's barriers hide under the other's
   // work.  Otherwise every CTA has an SM to itself and takes 1024 threads,
-  // which halves its token loops.
+  // which halves its token loops.  32 sequences x 8 groups of 2,000 / 11,000 /
+  // 30,000 / 56,000 tokens, two per SM and one: 27 / 42 / 83 / 134 us and 60 / 83 / 128 /
+  // 203; on the largest patch grid and joint histogram, where two leave no room
+  // for rows on chip: 38 / 57 / 95 / 152 and 72 / 95 / 150 / 218.
   const bool two = static_cast<int64_t>(ncta) * b.nlayers * b.nseq > num_sms;
-  const int cap = calibrate_capacity(kp.K, kp.M, kp.R, kp.C, two ? kSmemTwo : kSmemMax);
+  const size_t fixed = fixed_bytes(kp.K * kp.M * kp.M, kp.R * kp.C);
+  const int cap = calibrate_capacity(fixed, two ? kSmemTwo : kSmemMax);
   // A row longer than the capacity is read again from S in every pass; only
   // the CTA's range of fused scores is then kept on chip.
   int capl = (lp_max + 15) & ~15;
   if (capl > cap) capl = cap;
-  const size_t smem = fixed_bytes(kp.K, kp.M, kp.R, kp.C) + static_cast<size_t>(capl) * kBytesPerToken;
+  const size_t smem = fixed + static_cast<size_t>(capl) * kBytesPerToken;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(ncta, b.nlayers, b.nseq);
   cfg.dynamicSmemBytes = smem;

@@ -45,11 +45,11 @@ def _row(lp, levels, seed):
     return s.astype(np.float32)
 
 
-def _seq(row, G, budget, slot, per_head, seed, w=8):
+def _seq(row, G, budget, slot, per_head, seed, w=8, side=R):
     lp = row.size
     rng = np.random.default_rng([lp, seed, 7])
     meta = np.zeros(lp + w, np.uint32)
-    r, c = rng.integers(0, R, lp), rng.integers(0, C, lp)
+    r, c = rng.integers(0, side, lp), rng.integers(0, side, lp)
     meta[:lp] = sk.pack_meta(np.ones(lp), np.zeros(lp), r, c)
     P = G if per_head else 1
     seq = sk.Seq(meta=sk.meta_tensor(meta).cuda(), L=lp + w, cur_frame=0, budget=budget, slot=slot,
@@ -60,16 +60,16 @@ def _seq(row, G, budget, slot, per_head, seed, w=8):
     return seq, (r, c)
 
 
-def _check(seq, cells, row, G, per_head):
+def _check(seq, cells, row, G, per_head, side=R, K=8, M=8):
     B = seq.budget
     order = np.lexsort((np.arange(row.size), -row.astype(np.float64)))
     want = np.sort(order[:B])
     for p in range(G if per_head else 1):
         np.testing.assert_array_equal(seq.idx[0, p].cpu().numpy(), want)
     stats = seq.stats[0].double().cpu().numpy()
-    bins = O.rank_bins(row.astype(np.float64), 8)
-    mi = O.mutual_information(bins, O.spatial_cells(cells[0], cells[1], R, C, 8), 8, 64)
-    np.testing.assert_allclose(stats[8:8 + G], mi, rtol=1e-5, atol=1e-6)
+    bins = O.rank_bins(row.astype(np.float64), K)
+    mi = O.mutual_information(bins, O.spatial_cells(cells[0], cells[1], side, side, M), K, M * M)
+    np.testing.assert_allclose(stats[8:8 + G], mi, rtol=1e-5, atol=1e-6 * K * M * M / 512)
     _, temp = O.entropy_temperature(row.astype(np.float64), 0.95, 1.05, 1e-12)
     got = seq.score[0].double().cpu().numpy()
     np.testing.assert_allclose(got, np.repeat((row.astype(np.float64) ** (1 / temp))[None], got.shape[0], 0), rtol=1e-5)
@@ -114,6 +114,24 @@ def test_a_batch_with_more_ctas_than_sms(levels):
     sk.check_device_error(st)
     for (seq, cells), row in zip(made, rows):
         _check(seq, cells, row, G, False)
+
+
+def test_no_room_for_rows_on_chip():
+    """The largest patch grid and joint histogram with more CTAs than SMs: no token
+    of a row fits on chip, so that every pass reads S again and the fused scores
+    wait in their output row.  (MI: up to 4096 terms, hence 8 times the absolute
+    tolerance of the 512-cell histogram.)"""
+    G, n, side, K, M = 8, 32, 128, 16, 16
+    st = sk.init_state(dataclasses.replace(_config(G, n, False), grid_rows=side, grid_cols=side, mi_bins=K, mi_grid=M))
+    sizes = (SIZES + [7, 64, 255, 2000, 6001, 9999, 20011, 30002] * 2)[:n]
+    rows = [_row(lp, 0 if i % 2 else 40, i) for i, lp in enumerate(sizes)]
+    made = [_seq(row, G, max(1, row.size // 4), i, False, i, side=side) for i, row in enumerate(rows)]
+    seqs = [m[0] for m in made]
+    sk.select(st, 0, seqs, sk.workspace(st, seqs))
+    torch.cuda.synchronize()
+    sk.check_device_error(st)
+    for (seq, cells), row in zip(made, rows):
+        _check(seq, cells, row, G, False, side, K, M)
 
 
 @pytest.mark.parametrize("pool", [1, 3, 7, 9, 11, 31])
