@@ -116,6 +116,36 @@ def test_a_batch_with_more_ctas_than_sms(levels):
         _check(seq, cells, row, G, False)
 
 
+def _crowded_row(lp, n, equal, seed):
+    """lp scores spread over four octaves, n of them eight units of the last place
+    apart (all in one or two buckets of the first histogram), `equal` of these the same."""
+    rng = np.random.default_rng([lp, n, equal, seed])
+    s = np.exp2(rng.uniform(-4.0, 0.0, lp)).astype(np.float32)
+    crowd = np.float32(0.3).view(np.uint32) + 8 * np.arange(n, dtype=np.uint32)
+    crowd[n // 4:n // 4 + equal] = crowd[n // 4]
+    s[rng.permutation(lp)[:n]] = crowd.view(np.float32)
+    return s
+
+
+@pytest.mark.parametrize("equal", [0, 600, 3000], ids=["distinct", "600equal", "3000equal"])
+@pytest.mark.parametrize("lp", [5000, 14000, 56097])
+@pytest.mark.parametrize("G,per_head", [(1, False), (4, False), (4, True), (32, False)],
+                         ids=["G1", "G4", "G4_per_head", "G32"])
+def test_a_crowded_bucket_is_split_again(G, per_head, lp, equal):
+    """4000 scores in a bucket: its own key range gets a histogram, which is searched
+    for the B-th token; with many equal ones among them a second one, down to one key."""
+    st = sk.init_state(_config(G, 1, per_head))
+    row = _crowded_row(lp, 4000, equal, G)
+    above = int((row > np.float32(0.31)).sum())   # (the crowd lies between 0.3 and 0.301)
+    for B in (above + 1, above + 700, above + 2000, above + 3999):
+        sk.reset_seq(st, 0)
+        seq, cells = _seq(row, G, B, 0, per_head, G)
+        sk.select(st, 0, [seq], sk.workspace(st, [seq]))
+        torch.cuda.synchronize()
+        sk.check_device_error(st)
+        _check(seq, cells, row, G, per_head)
+
+
 def test_no_room_for_rows_on_chip():
     """The largest patch grid and joint histogram with more CTAs than SMs: no token
     of a row fits on chip, so that every pass reads S again and the fused scores
