@@ -282,9 +282,11 @@ starkv_status starkv_score_layer(starkv_state* st, int32_t layer, const starkv_s
  * device shares the one array and leaves its last contents there (nothing in
  * it has to start at zero): calls that may overlap on the GPU (different
  * streams, or threads without ordering) race on it and must not be issued.  A
- * batch whose scratch would exceed 16 MiB is rejected with
- * STARKV_ERR_UNSUPPORTED before any launch (about 1.8 MB per sequence at the
- * 5-screenshot UI-TARS shape); kernel timing must be off (it creates CUDA
+ * batch is rejected with STARKV_ERR_UNSUPPORTED before any launch when it counts
+ * more than 16 MiB by a fixed rule, an upper bound of what the kernels use: 2 KiB
+ * per (KV group, 128 past tokens begun) and 16 bytes per (KV group, past token), each
+ * sequence's tokens rounded up to 4 and its bytes to 256 (1.8 MB per sequence at
+ * the 5-screenshot UI-TARS shape); kernel timing must be off (it creates CUDA
  * events).  STARKV_ERR_CUDA if the array could not be reserved when the state
  * was created. */
 starkv_status starkv_score_layer_noalloc(starkv_state* st, int32_t layer, const starkv_seq* seqs,

@@ -1088,22 +1088,22 @@ extern "C" starkv_status starkv_score_layer_noalloc(starkv_state* st, int32_t la
   if (!st->noalloc_scratch)
     return set_error(STARKV_ERR_CUDA, "the static scratch is unavailable on device %d: %s", st->device,
                      st->noalloc_error.c_str());
-  // The limit counts the pass-1 partials and four unpooled rows per group (the
-  // kernels use one), so that the accepted batches do not depend on how pass 2
-  // splits its columns.
+  // The admission rule of the header: pass-1 partials and four float rows per group
+  // (the kernels need one), so that the accepted batches do not depend on how
+  // pass 2 splits its columns.
   const size_t G = st->cfg.n_kv_heads;
-  size_t need = 0, tiles = 0;
+  size_t counted = 0, tiles = 0;
   for (int i = 0; i < nseq; ++i) {
     const int lp = seqs[i].L - st->cfg.window;
     tiles += G * tiles_of(lp);
-    need += align256(G * 4 * raw_stride(lp) * sizeof(float));
+    counted += align256(G * 4 * raw_stride(lp) * sizeof(float));
   }
-  need = std::max<size_t>(need + align256(tiles * kMaxRows * sizeof(float2)), 256);
-  if (need > kNoAllocScratchBytes)
+  counted += align256(tiles * kMaxRows * sizeof(float2));
+  if (counted > kNoAllocScratchBytes)
     return set_error(STARKV_ERR_UNSUPPORTED,
-                     "this call needs %zu bytes of scratch; the static scratch holds %zu bytes: "
-                     "split the batch or use starkv_score_layer with a workspace",
-                     need, kNoAllocScratchBytes);
+                     "this batch counts %zu bytes against the %zu bytes of the static scratch (see the header for "
+                     "the rule): split it or use starkv_score_layer with a workspace",
+                     counted, kNoAllocScratchBytes);
   return run_stages(st, seqs, nseq, layer, 1, kScore | kPool, st->noalloc_scratch, kNoAllocScratchBytes,
                     static_cast<cudaStream_t>(stream));
 }

@@ -7,6 +7,8 @@ after call, with the window normalisers computed or supplied; it must leave the
 device's free memory unchanged, and it must refuse batches larger than its
 static scratch.  Collected last on purpose: it must pass alone in a fresh
 process and after every other test."""
+import re
+
 import numpy as np
 import pytest
 import torch
@@ -87,11 +89,19 @@ def test_noalloc_scoring_with_supplied_normalisers():
 def test_noalloc_rejects_a_batch_beyond_its_static_scratch():
     wl = syn.WORKLOADS["uitars_layer"]
     si = syn.make_sequence(wl)
-    n = 16  # ~1.8 MB of scratch each at this shape: more than 16 MiB together
+    n = 16  # counted at 1.8 MB each at this shape: more than 16 MiB together
     st = sk.init_state(H.gpu_config(wl, H.hyper(), max_seqs=n))
     seqs = [H.device_seq(si, wl, slot=i, with_score=False, with_stats=False).seq for i in range(n)]
     with pytest.raises(sk.StarkvError) as e:
         sk.score_layer_noalloc(st, 0, seqs)
     assert e.value.status == sk.ERR_UNSUPPORTED
     assert "static scratch" in str(e.value)
+    lp = si.L - wl.window
+    rule = n * wl.n_kv_heads * (-(-lp // 4) * 4 * 16 + -(-lp // 128) * 2048)
+    counted = int(re.search(r"counts (\d+) bytes", str(e.value)).group(1))   # (the message says by which rule, not "needs")
+    assert abs(counted - rule) < 256 * n
+    fits = (16 << 20) * n // counted
+    sk.score_layer_noalloc(st, 0, seqs[:fits])
+    torch.cuda.synchronize()
+    sk.check_device_error(st)
     st.close()
