@@ -5,7 +5,7 @@
 
 namespace starkv {
 
-constexpr int kAttnThreads = 512;   // 16 warps: TMA, MMA, 2 idle, 8 softmax, 4 V conversion
+constexpr int kAttnThreads = 512;   // 16 warps: 2 loaders, 2 MMA issuers, 8 softmax, 4 V conversion
 constexpr int kAttnUnitKeys = 64;   // keys per pipeline unit
 
 struct AttnSeq {

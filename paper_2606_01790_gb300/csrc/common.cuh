@@ -52,7 +52,7 @@ struct KParams {
   uint64_t wait_ns;    // bounded-wait limit
 };
 
-// One sequence of a launch, as the select / group-stats / compact kernels see it.
+// One sequence of a launch, as the pooling, calibration and compaction kernels see it.
 struct SeqView {
   const __nv_bfloat16* k;
   const __nv_bfloat16* v;

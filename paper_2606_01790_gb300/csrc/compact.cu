@@ -21,7 +21,8 @@ constexpr int kInFlight = 8;    // 16-byte accesses per lane in flight (16 rows 
 // 64 registers a thread and four blocks per SM (128 KB of loads in flight).  Left
 // to itself the compiler takes 76 registers, three blocks: 28 layers x 4 heads of
 // 14,032 / 56,128 tokens, 20 % kept, take 50 / 194 us that way and 48 / 185 us so,
-// which is the rate of a plain copy.  Five blocks (51 registers) spill: 56 / 203.
+// which is the rate of a plain copy.  Four still spill one register, five (51
+// registers) several: 56 / 203.
 constexpr int kBlocksPerSm = 4;
 
 __device__ __forceinline__ uint4 ld_stream(const uint4* p) {

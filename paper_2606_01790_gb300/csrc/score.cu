@@ -591,6 +591,10 @@ __global__ void __launch_bounds__(kScoreThreads, 1) k_score_lse(const __grid_con
 // them in order and stores the row.  No warp waits for another inside a piece,
 // and one row goes to memory instead of four.  A slot is written again at tile
 // j + 8, after every warp has released tile j + 6 and so read the slot before.
+// What orders a sum's store before its reader: the store precedes the warp's arrive
+// on t_empty for tile j + 1 (a release), the MMA issuer's wait on it acquires and
+// precedes its products of tile j + 3, whose tcgen05.commit completes the t_full
+// that the reader waits for.
 // The piece's last three tiles are stored after a barrier of the epilogue warps.
 // REV: the tiles go from the piece's last to its first.  `dst`: this thread's key of
 // the first, `left` keys of the row from it on.

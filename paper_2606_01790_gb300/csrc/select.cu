@@ -1005,6 +1005,9 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_calibrate(const __grid_consta
     int nlow = 0;                     // kept tokens of the lower-ranked CTAs, so far
     int bstar, rkb, ncb, coff, nown;
     bool ties = false;
+    // The loop's cluster barriers, and the one after it, stand behind conditions on
+    // ncb, lo and hi, which every CTA of the selection computes from the same
+    // exchanged counts and key ranges: all take the same way.
     for (;;) {
       // every warp for itself: the coarse bucket of the target on the summed
       // counts (four per lane), then its 32 buckets (one per lane)

@@ -182,8 +182,8 @@ def test_select_with_heavy_score_ties():
 
 
 def test_select_on_a_row_longer_than_shared_memory():
-    """20 screenshots (L_p = 56,096): the calibration kernel keeps the row's
-    keys in the workspace instead of shared memory."""
+    """20 screenshots (L_p = 56,096): the row's keys do not fit the calibration
+    kernel's shared memory, and every pass reads S again."""
     wl = syn.WORKLOADS["long_layer"]
     si = syn.make_sequence(wl)
     h = H.hyper(n_warmup=0, n_ramp=0)

@@ -98,8 +98,9 @@ def test_per_head_28_layer_step_at_the_benchmark_shape():
 
 
 def test_per_head_long_rows_beyond_shared_memory():
-    """20 screenshots + 2,048 text tokens (L_p = 56,096): the calibration keeps
-    its per-token arrays in the workspace instead of shared memory."""
+    """20 screenshots + 2,048 text tokens (L_p = 56,096): the row does not fit the
+    calibration kernel's shared memory; every pass reads S again, and the fused
+    scores wait in their output row."""
     wl = syn.WORKLOADS["long_layer"]
     si = syn.make_sequence(wl)
     h = H.hyper(n_warmup=0, n_ramp=0)

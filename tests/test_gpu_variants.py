@@ -60,9 +60,9 @@ def test_variant_matches_oracle_over_two_calls(variant, per_head):
 
 
 def test_variants_on_a_row_longer_than_shared_memory():
-    """20 screenshots + 2,048 text tokens (L_p = 56,096): the calibration keeps
-    its per-token arrays in the workspace; the decay and MI-span switches on
-    that path, over two calls."""
+    """20 screenshots + 2,048 text tokens (L_p = 56,096): the row does not fit the
+    calibration kernel's shared memory; the decay and MI-span switches on that
+    path, over two calls."""
     wl = syn.WORKLOADS["long_layer"]
     si = syn.make_sequence(wl)
     h = H.hyper(n_warmup=0, n_ramp=0, decay_mode=1, mi_span=1, aeb_mode=1)
